@@ -268,7 +268,9 @@ int tpm_compute_forces_noalloc(tpm_ctx *ctx, tpm_sys s, const uint32_t *active_i
  * sequence of batched calls can be captured in a CUDA graph.  All requests
  * of one call run in one persistent walk launch: resident warps take groups
  * of at most G consecutive (key-ordered) particles of any request from a
- * device work queue.  Open-boundary systems only.
+ * device work queue (groups of small systems, and of small requests whose
+ * particles lie apart, from a second queue, two particles a warp).
+ * Open-boundary systems only.
  */
 typedef struct tpm_plan tpm_plan;
 
@@ -277,7 +279,7 @@ typedef struct tpm_plan tpm_plan;
 #define TPM_BATCH_PRESORTED 1u
 
 /* Creates a plan for batches of at most max_ids ids in max_requests
- * requests (memory drawn from ctx's budget: about 40 B per id + 300 B per
+ * requests (memory drawn from ctx's budget: about 42 B per id + 300 B per
  * request).  Errors: TPM_EINVAL, TPM_EBUDGET, TPM_ECUDA. */
 int tpm_plan_create(tpm_ctx *ctx, int64_t max_ids, int64_t max_requests, tpm_plan **plan);
 

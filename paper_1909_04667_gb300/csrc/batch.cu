@@ -12,9 +12,11 @@
 //      (and, unless the caller says they already are, sorted by (request,
 //      key order)),
 //   2. each request is cut into groups of at most G consecutive particles
-//      (G is the plan's group size, chosen by tpm_plan_autotune),
+//      (G is the plan's group size, chosen by tpm_plan_autotune); those that
+//      get two particles a warp (small or sparse requests) are listed apart,
 //   3. one persistent walk launch lets resident warps take groups from a
-//      device work queue until it is empty.
+//      device work queue until it is empty, and another does the same for the
+//      groups listed apart, two particles an item.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -30,6 +32,7 @@ namespace {
 struct KeyReq {
     const uint32_t *rank;
     int64_t n;
+    int64_t rule;  // which of its groups get two particles a warp (batch_few_rule)
 };
 
 struct Plan {
@@ -41,8 +44,9 @@ struct Plan {
     uint64_t *keys = nullptr, *skeys = nullptr;
     uint32_t *vals = nullptr, *slot = nullptr, *sidx = nullptr;
     uint32_t *gcnt = nullptr, *goff = nullptr;
-    uint4 *groups = nullptr;
-    unsigned *ngroups = nullptr, *next = nullptr;
+    uint4 *groups = nullptr, *few = nullptr;
+    unsigned *ngroups = nullptr;
+    unsigned *next = nullptr, *few_next = nullptr, *nfew = nullptr;  // three words, cleared together
     int *err = nullptr;
     int64_t *off_dev = nullptr;
     KeyReq *kreq_dev = nullptr;
@@ -54,6 +58,10 @@ struct Plan {
     size_t cub_bytes = 0;
     cudaEvent_t staged = nullptr;  // host staging buffers may be rewritten once this has passed
     bool staged_pending = false;
+    // the groups that get two particles a warp are walked on a stream of the
+    // plan's own, beside the others: they fill the tail of that launch
+    cudaStream_t side = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 // Per requested id (one thread each, over all requests: one block per
@@ -109,16 +117,25 @@ __global__ void k_batch_gcount(const int64_t *__restrict__ off, int64_t n_req, i
 }
 
 // The group table of the persistent walk: (start, count, request, 0) for each
-// group of each request, from the scanned group counts; the total into ngroups.
-__global__ void k_batch_groups(const int64_t *__restrict__ off, const uint32_t *__restrict__ gcnt,
-                               const uint32_t *__restrict__ goff, int64_t n_req, int g, uint4 *__restrict__ groups,
-                               unsigned *__restrict__ ngroups) {
+// group of each request, from the scanned group counts; the total into
+// ngroups.  The groups that get two particles a warp go to a list of their
+// own (in any order: each is walked by itself) and are left in the table with
+// a count of 0.
+__global__ void k_batch_groups(const int64_t *__restrict__ off, const KeyReq *__restrict__ kr,
+                               const uint32_t *__restrict__ gcnt, const uint32_t *__restrict__ goff, int64_t n_req,
+                               int g, const uint32_t *__restrict__ sidx, uint4 *__restrict__ groups,
+                               unsigned *__restrict__ ngroups, uint4 *__restrict__ few, unsigned *__restrict__ nfew) {
     const int64_t r = blockIdx.x;
     const int64_t lo = off[r], hi = off[r + 1];
     const uint32_t base = goff[r], ng = gcnt[r];
+    const int rule = (int)kr[r].rule;
     for (uint32_t q = threadIdx.x; q < ng; q += blockDim.x) {
         const int64_t start = lo + (int64_t)q * g;
-        groups[base + q] = make_uint4((uint32_t)start, (uint32_t)min((int64_t)g, hi - start), (uint32_t)r, 0u);
+        const int count = (int)min((int64_t)g, hi - start);
+        const bool two = few_chunk(rule, sidx, start, count);
+        groups[base + q] = make_uint4((uint32_t)start, two ? 0u : (uint32_t)count, (uint32_t)r, 0u);
+        if (two)
+            few[atomicAdd(nfew, 1u)] = make_uint4((uint32_t)start, (uint32_t)count, (uint32_t)r, 0u);
     }
     if (r == n_req - 1 && threadIdx.x == 0)
         *ngroups = base + ng;
@@ -155,6 +172,14 @@ void release_plan(Plan *pl) {
         cudaFreeHost(pl->reqs_host);
     if (pl->staged)
         cudaEventDestroy(pl->staged);
+    if (pl->ev_fork)
+        cudaEventDestroy(pl->ev_fork);
+    if (pl->ev_join)
+        cudaEventDestroy(pl->ev_join);
+    if (pl->side)
+        cudaStreamDestroy(pl->side);
+    pl->ev_fork = pl->ev_join = nullptr;
+    pl->side = nullptr;
     pl->off_host = nullptr;
     pl->kreq_host = nullptr;
     pl->reqs_host = nullptr;
@@ -198,6 +223,7 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
         pl->staged_pending = false;
     }
     const size_t rb = batch_req_bytes();
+    bool any_few = false;  // some request has a rule
     {
         std::lock_guard<std::mutex> lk(c->mu);
         for (int64_t r = 0; r < n_req; r++) {
@@ -220,7 +246,10 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
                 set_error("request %lld uses the relative criterion: a_old is required", (long long)r);
                 return TPM_EINVAL;
             }
-            pl->kreq_host[r] = KeyReq{s->rank, s->n};
+            // groups of 64 have a walk of their own (two particles per lane)
+            const int rule = pl->group_size <= 32 ? batch_few_rule(s, offsets[r + 1] - offsets[r]) : kFewNone;
+            any_few = any_few || rule != kFewNone;
+            pl->kreq_host[r] = KeyReq{s->rank, s->n, rule};
             fill_batch_req(pl->reqs_host + r * rb, s, p);
             pl->off_host[r] = offsets[r];
         }
@@ -255,13 +284,24 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
     size_t b = pl->cub_bytes;
     TPM_CUDA(cub::DeviceScan::ExclusiveSum(pl->cub_tmp, b, pl->gcnt, pl->goff, (int)n_req, st));
     count_cub_call();
-    k_batch_groups<<<(unsigned)n_req, 128, 0, st>>>(pl->off_dev, pl->gcnt, pl->goff, n_req, g, pl->groups,
-                                                    pl->ngroups);
+    TPM_CUDA(cudaMemsetAsync(pl->next, 0, 3 * sizeof(unsigned), st));  // next, few_next, nfew
+    k_batch_groups<<<(unsigned)n_req, 128, 0, st>>>(pl->off_dev, pl->kreq_dev, pl->gcnt, pl->goff, n_req, g, pl->sidx,
+                                                    pl->groups, pl->ngroups, pl->few, pl->nfew);
     count_launch();
-    TPM_CUDA(cudaMemsetAsync(pl->next, 0, sizeof(unsigned), st));
     TPM_CUDA(cudaGetLastError());
-    return launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
-                             pl->slot, a_old, acc, pot, nint, pl->err, st);
+    if (!any_few)
+        return launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
+                                 pl->slot, a_old, acc, pot, nint, pl->err, st);
+    TPM_CUDA(cudaEventRecord(pl->ev_fork, st));
+    const int rc = launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
+                                     pl->slot, a_old, acc, pot, nint, pl->err, st);
+    TPM_CUDA(cudaStreamWaitEvent(pl->side, pl->ev_fork, 0));
+    const int rc_few = launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot,
+                                             a_old, acc, pot, nint, pl->err, pl->side);
+    // the caller's stream goes on when both are done, whatever the launches said
+    TPM_CUDA(cudaEventRecord(pl->ev_join, pl->side));
+    TPM_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
+    return rc != TPM_OK ? rc : rc_few;
 }
 
 }  // namespace
@@ -303,11 +343,14 @@ int tpm_plan_create(tpm_ctx *h, int64_t max_ids, int64_t max_requests, tpm_plan 
         (rc = pl->mem.get(&pl->vals, max_ids, st)) || (rc = pl->mem.get(&pl->slot, max_ids, st)) ||
         (rc = pl->mem.get(&pl->sidx, max_ids, st)) || (rc = pl->mem.get(&pl->gcnt, max_requests, st)) ||
         (rc = pl->mem.get(&pl->goff, max_requests, st)) || (rc = pl->mem.get(&pl->groups, pl->max_groups, st)) ||
-        (rc = pl->mem.get(&pl->ngroups, 1, st)) || (rc = pl->mem.get(&pl->next, 1, st)) ||
+        (rc = pl->mem.get(&pl->few, pl->max_groups, st)) || (rc = pl->mem.get(&pl->ngroups, 1, st)) ||
+        (rc = pl->mem.get(&pl->next, 3, st)) ||
         (rc = pl->mem.get(&pl->err, 1, st)) || (rc = pl->mem.get(&pl->off_dev, max_requests + 1, st)) ||
         (rc = pl->mem.get(&pl->kreq_dev, max_requests, st)) ||
         (rc = pl->mem.get(&pl->reqs_dev, max_requests * rb, st)))
         return fail(rc);
+    pl->few_next = pl->next + 1;
+    pl->nfew = pl->next + 2;
     size_t sort_b = 0, scan_b = 0;
     if (cub::DeviceRadixSort::SortPairs(nullptr, sort_b, pl->keys, pl->skeys, pl->vals, pl->slot, (int)max_ids, 0,
                                         end_bit_for(max_requests), st) != cudaSuccess ||
@@ -321,7 +364,10 @@ int tpm_plan_create(tpm_ctx *h, int64_t max_ids, int64_t max_requests, tpm_plan 
     if (cudaMallocHost(&pl->off_host, (max_requests + 1) * sizeof(int64_t)) != cudaSuccess ||
         cudaMallocHost(&pl->kreq_host, max_requests * sizeof(KeyReq)) != cudaSuccess ||
         cudaMallocHost(&pl->reqs_host, max_requests * rb) != cudaSuccess ||
-        cudaEventCreateWithFlags(&pl->staged, cudaEventDisableTiming) != cudaSuccess) {
+        cudaEventCreateWithFlags(&pl->staged, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&pl->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+        cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking) != cudaSuccess) {
         set_error("pinned staging allocation failed");
         return fail(TPM_ECUDA);
     }

@@ -252,7 +252,23 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
 // request, 0) over the sorted active list; group_size 64 takes the walk with
 // two particles per lane (else groups of at most 32, one per lane);
 // stack_depth is the candidate-stack capacity of the walk (128, 192 or 256).
+// The groups that get two particles a warp (few_chunk, by the rule of their
+// request: batch_few_rule for its number of ids) have a list and a launch of
+// their own.
+enum { kFewNone = 0, kFewSparse = 1, kFewAll = 2 };
+constexpr uint32_t kSparseSpan = 8;
+#ifdef __CUDACC__
+__device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__ sidx, int64_t g0, int gcount) {
+    if (rule != kFewSparse)
+        return rule == kFewAll;
+    return sidx && sidx[g0 + gcount - 1] - sidx[g0] >= kSparseSpan * (uint32_t)gcount;
+}
+#endif
 size_t batch_req_bytes();
+int batch_few_rule(const System *s, int64_t n_ids);
+int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
+                          unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
+                          float *pot, uint32_t *nint, int *err, cudaStream_t st);
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p);
 int launch_walk_batch(Ctx *c, int group_size, int stack_depth, const void *reqs, const uint4 *groups,
                       const unsigned *n_groups, unsigned *next, const uint32_t *sidx, const uint32_t *slot,

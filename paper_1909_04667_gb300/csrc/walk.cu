@@ -1368,6 +1368,8 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
 }
 
 
+#include "walk_few.cuh"
+
 // Walks a chunk of consecutive active particles: in one frame, or, when it
 // is spread out (chunk_cuts), run by run, each run in its own frame.
 template <bool PERIODIC, bool RELATIVE, bool TREEPM, bool VARH, class SH>
@@ -1391,22 +1393,24 @@ __device__ __forceinline__ void walk_runs_of_chunk(const TreeView &T, const Walk
     }
 }
 
-// One warp per group of `gsize` consecutive active particles.  Seven blocks
+// One warp per group of 32 consecutive active particles.  Seven blocks
 // of four warps per SM: the register cap (72) that keeps the paired FP32
 // sweeps and decisions free of spills (measured against caps of 64 and none).
 template <bool PERIODIC, bool RELATIVE, bool TREEPM, bool VARH>
 __global__ void __launch_bounds__(kGroupWarps * 32, 7)
     k_walk_group(TreeView T, const uint32_t *__restrict__ sidx, const uint32_t *__restrict__ slot,
-                 const float *__restrict__ a_old, int64_t n_act, int gsize, WalkConsts k, float *__restrict__ acc,
+                 const float *__restrict__ a_old, int64_t n_act, int rule, WalkConsts k, float *__restrict__ acc,
                  float *__restrict__ pot, uint32_t *__restrict__ nint, int accumulate, int *__restrict__ err) {
     using SH = GroupSharedT<kStackCap, VARH, PERIODIC>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SH &sh = reinterpret_cast<SH *>(smem_raw)[threadIdx.x >> 5];
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t g0 = warp * gsize;
+    const int64_t g0 = warp * 32;
     if (g0 >= n_act)
         return;  // whole warp
-    const int gcount = (int)min((int64_t)gsize, n_act - g0);
+    const int gcount = (int)min((int64_t)32, n_act - g0);
+    if (!PERIODIC && few_chunk(rule, sidx, g0, gcount))
+        return;  // walked two targets a warp
     walk_runs_of_chunk<PERIODIC, RELATIVE, TREEPM, VARH>(T, k, sh, sidx, slot, g0, gcount, a_old, acc, pot, nint,
                                                          accumulate, err);
 }
@@ -1947,6 +1951,8 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 7)
         if (g >= total)
             break;
         const uint4 G = groups[g];
+        if (G.y == 0u)
+            continue;  // walked two particles a warp
         {
             static_assert(sizeof(BatchReq) % 4 == 0, "request records copy as words");
             const uint32_t *src = reinterpret_cast<const uint32_t *>(&reqs[G.z]);
@@ -1961,6 +1967,46 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 7)
         else
             walk_runs_of_chunk<PERIODIC, false, TREEPM, false>(R.T, R.k, sh, sidx, slot, G.x, (int)G.y, a_old, acc,
                                                                pot, nint, 0, err);
+        __syncwarp();
+    }
+}
+
+// The groups of a batch that get two particles a warp: resident warps take
+// items of two particles from their own queue.
+__global__ void __launch_bounds__(kFewWarps * 32)
+    k_walk_batch_few(const BatchReq *__restrict__ reqs, const uint4 *__restrict__ groups,
+                     const unsigned *__restrict__ n_groups, int items, unsigned *__restrict__ next,
+                     const uint32_t *__restrict__ sidx, const uint32_t *__restrict__ slot,
+                     const float *__restrict__ a_old, float *__restrict__ acc, float *__restrict__ pot,
+                     uint32_t *__restrict__ nint, int *__restrict__ err) {
+    __shared__ FewShared shared[kFewWarps];
+    __shared__ __align__(16) BatchReq breq[kFewWarps];
+    FewShared &sh = shared[threadIdx.x >> 5];
+    BatchReq &R = breq[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const unsigned long long total = (unsigned long long)*n_groups * items;
+    for (;;) {
+        unsigned g = 0;
+        if (lane == 0)
+            g = atomicAdd(next, 1u);
+        g = __shfl_sync(0xffffffffu, g, 0);
+        if (g >= total)
+            break;
+        const uint4 G = groups[g / items];
+        const int lo = 2 * (int)(g % items), hi = min(lo + 2, (int)G.y);
+        if (lo >= hi)
+            continue;
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(&reqs[G.z]);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&R);
+        for (int w = lane; w < (int)(sizeof(BatchReq) / 4); w += 32)
+            dst[w] = src[w];
+        __syncwarp();
+        if (R.relative)
+            few_walk_chunk<true, false, false>(R.T, R.k, sh, sidx, slot, G.x, (int)G.y, lo, hi, a_old, acc, pot, nint,
+                                               0, err);
+        else
+            few_walk_chunk<false, false, false>(R.T, R.k, sh, sidx, slot, G.x, (int)G.y, lo, hi, a_old, acc, pot, nint,
+                                                0, err);
         __syncwarp();
     }
 }
@@ -2006,7 +2052,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 5)
 }
 
 template <bool P, bool R, bool T, bool V>
-void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, int *err, int num_sms,
+void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, int rule, int *err, int num_sms,
             cudaStream_t st) {
     const int64_t warps = (r.n_act + 31) / 32;
     if (lanes) {
@@ -2020,10 +2066,20 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
     const size_t smem = kGroupWarps * sizeof(GroupSharedT<kStackCap, V, P>);
     TreeView tv{s->bcen, s->bcom, s->blink, s->spart, s->psoft, s->bsoft, s->key,
                 s->perm, s->pos,  s->x0[0], s->x0[1],  s->x0[2], s->L0};
+    if constexpr (!P) {
+        if (rule != kFewNone) {
+            const int64_t blocks = (r.n_act + 2 * kFewWarps - 1) / (2 * kFewWarps);
+            k_walk_few<R, T, V><<<(unsigned)blocks, kFewWarps * 32, 0, st>>>(
+                tv, r.sorted_idx, r.slot, r.a_old, r.n_act, rule, k, r.acc, r.pot, r.nint, r.accumulate, err);
+            count_launch();
+            if (rule == kFewAll)
+                return;
+        }
+    }
     if (!lanes) {
         const int64_t blocks = (warps + kGroupWarps - 1) / kGroupWarps;
         k_walk_group<P, R, T, V><<<(unsigned)blocks, kGroupWarps * 32, smem, st>>>(
-            tv, r.sorted_idx, r.slot, r.a_old, r.n_act, 32, k, r.acc, r.pot, r.nint, r.accumulate, err);
+            tv, r.sorted_idx, r.slot, r.a_old, r.n_act, rule, k, r.acc, r.pot, r.nint, r.accumulate, err);
         count_launch();
     } else if constexpr (!P) {
         // the lane walk hands spread-out chunks to the group walk: their runs
@@ -2086,6 +2142,29 @@ void set_ewald(WalkConsts &k, const System *s, const float4 *tab, float phi0) {
 }  // namespace
 
 size_t batch_req_bytes() { return sizeof(BatchReq); }
+
+int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
+                          unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
+                          float *pot, uint32_t *nint, int *err, cudaStream_t st) {
+    static int blocks_per_sm = 0;  // resident blocks (one persistent wave)
+    if (!blocks_per_sm) {
+        int b = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_walk_batch_few, kFewWarps * 32, 0) != cudaSuccess ||
+            b < 1)
+            b = 1;
+        blocks_per_sm = b;
+    }
+    k_walk_batch_few<<<(unsigned)(c->num_sms * blocks_per_sm), kFewWarps * 32, 0, st>>>(
+        static_cast<const BatchReq *>(reqs), groups, n_groups, (group_size + 1) / 2, next, sidx, slot, a_old, acc, pot,
+        nint, err);
+    count_launch();
+    TPM_CUDA(cudaGetLastError());
+    return TPM_OK;
+}
+
+int batch_few_rule(const System *s, int64_t n_ids) {
+    return walk_override() == 0 ? few_rule(s, n_ids, true) : kFewNone;
+}
 
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p) {
     BatchReq r{};
@@ -2203,22 +2282,28 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
         set_error("per-particle softening is available with open boundaries");
         return TPM_EINVAL;
     }
+    int rule = kFewNone;
+    if (ov == 0 && !per) {
+        rule = few_rule(s, r.n_act, !tpm && !varh);
+        if (rule == kFewSparse && !r.sorted_idx)
+            rule = kFewNone;  // all particles: no chunk is sparse
+    }
     if (!per && !tpm)
-        rel ? (varh ? launch<false, true, false, true>(s, r, k, lanes, err, c->num_sms, st)
-                    : launch<false, true, false, false>(s, r, k, lanes, err, c->num_sms, st))
-            : (varh ? launch<false, false, false, true>(s, r, k, lanes, err, c->num_sms, st)
-                    : launch<false, false, false, false>(s, r, k, lanes, err, c->num_sms, st));
+        rel ? (varh ? launch<false, true, false, true>(s, r, k, lanes, rule, err, c->num_sms, st)
+                    : launch<false, true, false, false>(s, r, k, lanes, rule, err, c->num_sms, st))
+            : (varh ? launch<false, false, false, true>(s, r, k, lanes, rule, err, c->num_sms, st)
+                    : launch<false, false, false, false>(s, r, k, lanes, rule, err, c->num_sms, st));
     else if (!per && tpm)
-        rel ? (varh ? launch<false, true, true, true>(s, r, k, lanes, err, c->num_sms, st)
-                    : launch<false, true, true, false>(s, r, k, lanes, err, c->num_sms, st))
-            : (varh ? launch<false, false, true, true>(s, r, k, lanes, err, c->num_sms, st)
-                    : launch<false, false, true, false>(s, r, k, lanes, err, c->num_sms, st));
+        rel ? (varh ? launch<false, true, true, true>(s, r, k, lanes, rule, err, c->num_sms, st)
+                    : launch<false, true, true, false>(s, r, k, lanes, rule, err, c->num_sms, st))
+            : (varh ? launch<false, false, true, true>(s, r, k, lanes, rule, err, c->num_sms, st)
+                    : launch<false, false, true, false>(s, r, k, lanes, rule, err, c->num_sms, st));
     else if (tpm)
-        rel ? launch<true, true, true, false>(s, r, k, lanes, err, c->num_sms, st)
-            : launch<true, false, true, false>(s, r, k, lanes, err, c->num_sms, st);
+        rel ? launch<true, true, true, false>(s, r, k, lanes, rule, err, c->num_sms, st)
+            : launch<true, false, true, false>(s, r, k, lanes, rule, err, c->num_sms, st);
     else
-        rel ? launch<true, true, false, false>(s, r, k, lanes, err, c->num_sms, st)
-            : launch<true, false, false, false>(s, r, k, lanes, err, c->num_sms, st);
+        rel ? launch<true, true, false, false>(s, r, k, lanes, rule, err, c->num_sms, st)
+            : launch<true, false, false, false>(s, r, k, lanes, rule, err, c->num_sms, st);
     TPM_CUDA(cudaGetLastError());
     return TPM_OK;
 }
