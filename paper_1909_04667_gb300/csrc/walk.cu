@@ -279,8 +279,23 @@ __device__ __forceinline__ void append_runs(unsigned cut, int64_t g0, int gcount
     }
 }
 
-template <bool PERIODIC, bool RELATIVE, bool TREEPM, bool VARH>
-__global__ void __launch_bounds__(kWalkThreads)
+// The lane walk.  SPLIT: a block serves one chunk, and its warps share the
+// pre-order node array: it is cut into kSplitSegments equal segments per warp,
+// dealt round robin, and a warp takes the terms of the nodes of its segments.
+// To start inside the array it passes the subtrees that end before the
+// segment and decides the segment's ancestors (at most one a level) without
+// taking terms from them.  The warps' sums are added in order of the warps.
+// Used for the Ewald tree, whose walks visit most of the array (a particle of
+// the linear box sums thousands of terms, each with a gather from the
+// correction table): with one warp a chunk a 32^3 box has 1024 warps, and the
+// longest of them was the time of the call (9.9 ms of 10.6; 3.9 with 8 warps a
+// chunk, where the gathers of the correction table bound it).
+constexpr int kSplitSegments = 16;  // per warp: 4 / 8 / 16 / 32 took 4.08 / 4.02 / 3.88 / 3.82 ms (32^3 box, 8 warps)
+constexpr int kSplitMax = 16;  // warps per chunk
+constexpr size_t kSplitBytes = 2 * sizeof(float4) + sizeof(uint32_t);  // shared memory per thread
+
+template <bool PERIODIC, bool RELATIVE, bool TREEPM, bool VARH, bool SPLIT>
+__global__ void __launch_bounds__(SPLIT ? 32 * kSplitMax : kWalkThreads)
     k_walk(const float4 *__restrict__ ncen, const float4 *__restrict__ ncom, const int4 *__restrict__ nlink,
            const float4 *__restrict__ spart, const uint64_t *__restrict__ key, const uint32_t *__restrict__ perm,
            const double *__restrict__ pos, double x0, double y0, double z0, double L0, int nnodes,
@@ -290,7 +305,8 @@ __global__ void __launch_bounds__(kWalkThreads)
            uint2 *__restrict__ runs, unsigned *__restrict__ nruns) {
     constexpr bool EWALD = PERIODIC && !TREEPM;  // periodic tree without the mesh
     const int lane = threadIdx.x & 31;
-    const int64_t g0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane);
+    const int warps = SPLIT ? (int)(blockDim.x >> 5) : 1, w = SPLIT ? (int)(threadIdx.x >> 5) : 0;
+    const int64_t g0 = SPLIT ? (int64_t)blockIdx.x * 32 : ((int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane);
     if (g0 >= n_act)
         return;  // the whole warp leaves together
     if (!PERIODIC && !k.plain) {  // spread-out chunks are walked in runs by the group walk
@@ -333,9 +349,21 @@ __global__ void __launch_bounds__(kWalkThreads)
     float ax = 0.f, ay = 0.f, az = 0.f, ph = 0.f;
     float4 ec = make_float4(0.f, 0.f, 0.f, 0.f);  // compensation of the Ewald sums
     uint32_t cnt = 0;
+    for (int seg = w; seg < (SPLIT ? warps * kSplitSegments : 1); seg += warps) {
+    const int segs = warps * kSplitSegments;
+    const int first = SPLIT ? (int)((int64_t)nnodes * seg / segs) : 0;
+    const int last = SPLIT ? (int)((int64_t)nnodes * (seg + 1) / segs) : nnodes;
     int skip_until = valid ? 0 : 0x7fffffff;
     int n = 0;
-    while (n < nnodes) {
+    while (n < last) {
+        if (SPLIT && n < first) {
+            const int end = __ldg(&nlink[n].x);
+            if (end <= first) {  // a subtree before the segment
+                n = end;
+                continue;
+            }
+        }
+        const bool own = !SPLIT || n >= first;
         const float4 C = __ldg(&ncen[n]);
         const float4 O = __ldg(&ncom[n]);
         const int4 Lk = __ldg(&nlink[n]);
@@ -376,7 +404,7 @@ __global__ void __launch_bounds__(kWalkThreads)
         }
         const bool open = act && !far && (guard || crit);
         if (act && !open) {
-            if (!far) {
+            if (!far && own) {
                 if (EWALD)
                     ewald_pair_term(rx, ry, rz, r2, O.w, k, ax, ay, az, ph, ec);
                 else if (VARH)
@@ -420,6 +448,31 @@ __global__ void __launch_bounds__(kWalkThreads)
             }
         }
         n = Lk.x;
+    }
+    }
+    if (SPLIT) {
+        // the parts of the chunk's warps, added in FP64 (the parts are of the
+        // size of the whole attraction, the total a small difference)
+        extern __shared__ __align__(16) unsigned char smem_raw[];
+        float4 *part = reinterpret_cast<float4 *>(smem_raw), *rest = part + 32 * warps;
+        uint32_t *cnts = reinterpret_cast<uint32_t *>(rest + 32 * warps);
+        part[threadIdx.x] = make_float4(ax, ay, az, ph);
+        rest[threadIdx.x] = ec;
+        cnts[threadIdx.x] = cnt;
+        __syncthreads();
+        if (w)
+            return;
+        double sx = 0.0, sy = 0.0, sz = 0.0, sp = 0.0;
+        cnt = 0;
+        for (int v = 0; v < warps; v++) {
+            const float4 a = part[32 * v + lane], c = rest[32 * v + lane];
+            sx += (double)a.x - (double)c.x;
+            sy += (double)a.y - (double)c.y;
+            sz += (double)a.z - (double)c.z;
+            sp += (double)a.w - (double)c.w;
+            cnt += cnts[32 * v + lane];
+        }
+        ax = (float)sx, ay = (float)sy, az = (float)sz, ph = (float)sp;
     }
     if (!valid)
         return;
@@ -2056,12 +2109,29 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
             cudaStream_t st) {
     const int64_t warps = (r.n_act + 31) / 32;
     if (lanes) {
-        const int64_t blocks = (warps * 32 + kWalkThreads - 1) / kWalkThreads;
-        k_walk<P, R, T, V><<<(unsigned)blocks, kWalkThreads, 0, st>>>(
-            s->ncen, s->ncom, s->nlink, s->spart, s->key, s->perm, s->pos, s->x0[0], s->x0[1], s->x0[2], s->L0,
-            (int)s->nnodes, s->psoft, s->nsoft, r.sorted_idx, r.slot, r.a_old, r.n_act, k, r.acc, r.pot, r.nint,
-            r.accumulate, r.runs, r.nruns);
-        count_launch();
+        auto walk = [&](auto kernel, int64_t blocks, int threads, size_t smem) {
+            kernel<<<(unsigned)blocks, threads, smem, st>>>(
+                s->ncen, s->ncom, s->nlink, s->spart, s->key, s->perm, s->pos, s->x0[0], s->x0[1], s->x0[2], s->L0,
+                (int)s->nnodes, s->psoft, s->nsoft, r.sorted_idx, r.slot, r.a_old, r.n_act, k, r.acc, r.pot, r.nint,
+                r.accumulate, r.runs, r.nruns);
+            count_launch();
+        };
+        // the Ewald tree: warps per chunk until they fill the chip (64 registers:
+        // 32 warps an SM), twice over with the relative criterion, whose walks
+        // are long and uneven (32^3 box, 1024 chunks, 1 / 4 / 8 / 16 warps:
+        // 10.3 / 4.5 / 3.9 / 3.6 ms; 40^3, 2000 chunks: 13.8 / 7.7 / 7.0 / 6.9);
+        // the short ones of the geometric criterion lose more to the starts of
+        // segments (theta = 0.7, 40^3, 1 / 2 / 4 / 8: 1.25 / 1.15 / 1.26 / 1.35 ms)
+        int split = 1;
+        if (P && !T)
+            while (split < kSplitMax && 2 * split * warps <= (R ? 64 : 32) * (int64_t)num_sms)
+                split *= 2;
+        if constexpr (P && !T) {
+            if (split > 1)
+                walk(k_walk<P, R, T, V, true>, warps, 32 * split, 32 * split * kSplitBytes);
+        }
+        if (split == 1)
+            walk(k_walk<P, R, T, V, false>, (warps * 32 + kWalkThreads - 1) / kWalkThreads, kWalkThreads, 0);
     }
     const size_t smem = kGroupWarps * sizeof(GroupSharedT<kStackCap, V, P>);
     TreeView tv{s->bcen, s->bcom, s->blink, s->spart, s->psoft, s->bsoft, s->key,
