@@ -18,8 +18,9 @@
 //      ranges, skip indices and parents follow from searches in the sorted
 //      keys.  No level-by-level passes and no host round trip but one (the
 //      node count, to size the node tables)
-//   4. FP64 masses and mass-weighted positions summed bottom-up in one pass,
-//      children in ascending octant order and a leaf's particles in sorted
+//   4. FP64 masses and mass-weighted positions summed bottom-up, stretches of
+//      the key order by their own blocks and what reaches past them
+//      afterwards, children in ascending octant order and a leaf's particles in sorted
 //      order, with explicit round-to-nearest operations (no contraction), so
 //      the result is the same bit for bit on any correct implementation of
 //      that order
@@ -29,7 +30,6 @@
 //      -- three 16-byte records loaded with one vector load each -- and per
 //      sorted particle its position relative to its leaf centre plus mass.
 #include <cub/cub.cuh>
-#include <cuda/atomic>
 
 #include <algorithm>
 #include <climits>
@@ -112,50 +112,57 @@ __device__ void root_cube(BuildState *__restrict__ st, int periodic, double box,
 
 // Copies positions and masses into the system, applies the periodic shift and
 // wrap, checks finiteness and ranges (and the per-particle softening lengths,
-// if any), and reduces the bounding box; the last block to finish computes the
-// root cube from it.
+// if any), and reduces the bounding box (open boundaries); the last block to
+// finish computes the root cube from it.
 __global__ void k_prepare(const double *__restrict__ pin, const float *__restrict__ mass_in,
                           const float *__restrict__ hsoft, int64_t n, int periodic, double box, double s0, double s1,
                           double s2, double *__restrict__ pout, float *__restrict__ mout,
                           BuildState *__restrict__ state) {
     long long *bbox = state->bbox;
-    int *bad = &state->bad;
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    long long lo[3], hi[3];
-    bool have = i < n;
-    if (have) {
-        const double sh[3] = {s0, s1, s2};
+    long long lo[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, hi[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
+    int bad = 0;
+    // comparisons on the bits: non-negative doubles order like integers, and
+    // FP64 instructions (comparisons too) are what bounds this kernel
+    const uint64_t box_bits = (uint64_t)__double_as_longlong(box), inf_bits = 0x7ffull << 52, minus0 = 1ull << 63;
+    const double sh[3] = {__dmul_rn(s0, box), __dmul_rn(s1, box), __dmul_rn(s2, box)};
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             double v = pin[3 * i + a];
-            if (!isfinite(v))
-                atomicOr(bad, 1);
+            const uint64_t vb = (uint64_t)__double_as_longlong(v);
+            bad |= (vb & inf_bits) == inf_bits ? 1 : 0;
             if (periodic) {
-                if (!(v >= 0.0 && v < box))
-                    atomicOr(bad, 2);
-                v = __dadd_rn(v, __dmul_rn(sh[a], box));
-                if (v >= box)
+                bad |= vb < box_bits || vb == minus0 ? 0 : 2;
+                v = __dadd_rn(v, sh[a]);
+                if ((uint64_t)__double_as_longlong(v) >= box_bits)
                     v = __dsub_rn(v, box);
+            } else {
+                lo[a] = min(lo[a], ordered_bits(v));
+                hi[a] = max(hi[a], ordered_bits(v));
             }
             pout[3 * i + a] = v;
-            lo[a] = hi[a] = ordered_bits(v);
         }
-        float m = mass_in[i];
-        if (!(m > 0.0f) || !isfinite(m))
-            atomicOr(bad, 4);
+        const float m = mass_in[i];
+        bad |= m > 0.0f && isfinite(m) ? 0 : 4;
         mout[i] = m;
         if (hsoft) {
             const float h = hsoft[i];
-            if (!(h > 0.0f) || !isfinite(h))
-                atomicOr(bad, 8);
+            bad |= h > 0.0f && isfinite(h) ? 0 : 8;
         }
+    }
+    if (bad)
+        atomicOr(&state->bad, bad);
+    if (periodic) {  // the root is the box
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            root_cube(state, periodic, box, s0, s1, s2);
+        return;
     }
     // warp-level min / max, then one atomic per block
     __shared__ long long red[2][3][32];
     const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-        long long l = have ? lo[a] : LLONG_MAX, h = have ? hi[a] : LLONG_MIN;
+        long long l = lo[a], h = hi[a];
         for (int o = 16; o > 0; o >>= 1) {
             l = min(l, __shfl_xor_sync(0xffffffffu, l, o));
             h = max(h, __shfl_xor_sync(0xffffffffu, h, o));
@@ -205,16 +212,16 @@ __device__ __forceinline__ uint32_t compact3(uint64_t v) {
     return (uint32_t)v;
 }
 
-// floor(v) clamped to [0, 2^21 - 1], read off the bits of v (integer
-// operations only: FP64 arithmetic is scarce on this GPU).  v = m 2^(e - 52)
-// with the 53-bit significand m; for 1 <= v < 2^21 the integer part is
-// m >> (52 - e); negative v (sign bit set) and v < 1 give 0, v >= 2^21 (and
-// non-finite v) the largest coordinate.
-__device__ __forceinline__ uint32_t cell_coord(double v) {
+// floor(v 2^shift) clamped to [0, 2^21 - 1], read off the bits of v (integer
+// operations only: FP64 arithmetic is scarce on this GPU).  With v 2^shift =
+// m 2^(e - 52), m the 53-bit significand, the integer part for 1 <= v 2^shift
+// < 2^21 is m >> (52 - e); negative v (sign bit set) and values below 1 give
+// 0, values from 2^21 on (and non-finite v) the largest coordinate.
+__device__ __forceinline__ uint32_t cell_coord(double v, int shift) {
     const long long b = __double_as_longlong(v);
-    if (b < 0)
+    if (b < 0 || b < (1ll << 52))  // negative, zero or denormal
         return 0u;
-    const int e = (int)(b >> 52) - 1023;
+    const int e = (int)(b >> 52) - 1023 + shift;
     if (e < 0)
         return 0u;
     if (e >= kMaxLevel)
@@ -229,32 +236,30 @@ __global__ void k_keys(const double *__restrict__ pos, int64_t n, const BuildSta
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n)
         return;
+    // One FP64 operation per coordinate (they bound this kernel): with open
+    // boundaries the scale is a power of two, 2^shift, and the product an
+    // addition to the exponent; a periodic box has its corner at 0.
     const double o[3] = {st->x0[0], st->x0[1], st->x0[2]};
     const double scale = st->scale;
-    uint64_t k = 0;
+    const uint64_t sb = (uint64_t)__double_as_longlong(scale);
+    // (roots below 2^-580 keep the product: their coordinates may be denormal)
+    const bool pow2 = (sb & 0xfffffffffffffull) == 0ull && sb < (1623ull << 52);
+    const int shift = pow2 ? (int)(sb >> 52) - 1023 : 0;
+    double v[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]};
+    if (o[0] != 0.0 || o[1] != 0.0 || o[2] != 0.0) {
 #pragma unroll
-    for (int a = 0; a < 3; a++)
-        k |= spread3(cell_coord(__dmul_rn(__dsub_rn(pos[3 * i + a], o[a]), scale))) << a;
+        for (int a = 0; a < 3; a++)
+            v[a] = __dsub_rn(v[a], o[a]);
+    }
+    if (!pow2) {
+#pragma unroll
+        for (int a = 0; a < 3; a++)
+            v[a] = __dmul_rn(v[a], scale);
+    }
+    const uint64_t k = spread3(cell_coord(v[0], shift)) | spread3(cell_coord(v[1], shift)) << 1 |
+                       spread3(cell_coord(v[2], shift)) << 2;
     key[i] = k;
     idx[i] = (uint32_t)i;
-}
-
-// Inverse permutation, and positions and masses gathered into key order for
-// the passes over leaves.
-__global__ void k_rank(const uint32_t *__restrict__ perm, int64_t n, const double *__restrict__ pos,
-                       const float *__restrict__ mass, const float *__restrict__ hsoft, uint32_t *__restrict__ rank,
-                       double *__restrict__ spos, float *__restrict__ smass, float *__restrict__ psoft) {
-    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= n)
-        return;
-    const uint32_t j = perm[s];
-    rank[j] = (uint32_t)s;
-    spos[3 * s] = pos[3 * j];
-    spos[3 * s + 1] = pos[3 * j + 1];
-    spos[3 * s + 2] = pos[3 * j + 2];
-    smass[s] = mass[j];
-    if (hsoft)  // per-particle softening, in key order (checked by k_prepare)
-        psoft[s] = hsoft[j];
 }
 
 // Deepest level whose cell holds both keys (kMaxLevel when they are equal).
@@ -354,168 +359,6 @@ __global__ void k_node_counts(const uint64_t *__restrict__ key, int64_t n, int B
     cnt[i] = (uint32_t)max(D - lp, 0);
 }
 
-// Pre-order node arrays of the build.
-struct NodeArrays {
-    uint32_t *first, *count, *skip, *parent, *nchild, *arrive, *order;
-    uint8_t *level;
-    uint64_t *prefix;
-};
-
-// K3c. The nodes whose first particle is sorted particle i, from the top
-// down: particle range (the cell's end found by searching the sorted keys),
-// skip index (the first node of the particle just past the cell), key prefix,
-// parent (the node above with the same first particle, else the cell found by
-// searching downwards) and, by one atomic per node, the parent's child count.
-__global__ void k_nodes(const uint64_t *__restrict__ key, int64_t n, const uint32_t *__restrict__ base,
-                        const uint8_t *__restrict__ top_level, const uint8_t *__restrict__ leaf_level, NodeArrays t) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n)
-        return;
-    const uint32_t p0 = base[i], nc = base[i + 1] - p0;
-    if (nc == 0)
-        return;
-    const uint32_t total = base[n];
-    const int l0 = top_level[i];
-    const uint64_t ki = key[i];
-    uint32_t end = (uint32_t)n;
-    for (uint32_t k = 0; k < nc; k++) {
-        const int l = l0 + (int)k;
-        const uint32_t p = p0 + k;
-        const int sh = 3 * (kMaxLevel - l);
-        const uint64_t pre = ki >> sh;
-        end = search_up(key, (uint32_t)i + 1, end, (pre + 1) << sh);  // cells nest: the end only shrinks
-        t.first[p] = (uint32_t)i;
-        t.count[p] = end - (uint32_t)i;
-        t.skip[p] = end < n ? base[end] : total;
-        t.level[p] = (uint8_t)l;
-        t.prefix[p] = pre;
-        t.order[p] = p;
-        uint32_t par = 0;
-        if (l > 0) {
-            if (k > 0) {
-                par = p - 1;
-            } else {
-                const uint32_t f = search_down(key, (uint32_t)i, (pre >> 3) << (sh + 3));
-                par = base[f] + (uint32_t)(l - 1 - top_level[f]);
-            }
-            atomicAdd(&t.nchild[par], 1u);
-        }
-        t.parent[p] = par;
-    }
-}
-
-// K4: FP64 monopoles in one pass, bottom-up.  Each leaf sums its particles in
-// sorted order; then the last child of a node to finish (counted with an
-// atomic on the parent) sums the node's children in ascending octant order,
-// and so on up to the root.  Sums are stored by breadth-first index, where a
-// node's children are contiguous, so the children's sums load independently.
-// Explicit round-to-nearest adds / muls, so every sum has the same fixed
-// order and value whichever thread computes it.  The climb is a chain of
-// dependent memory round trips, so each step loads the links it needs next
-// (parent, child count, breadth-first indices: read-only here) before its
-// atomic, and a leaf loads its particles four at a time before summing them.
-__global__ void k_multipole(NodeArrays t, int64_t total, const uint32_t *__restrict__ pre2bfs,
-                            const double *__restrict__ spos, const float *__restrict__ smass, double *__restrict__ M,
-                            double *__restrict__ S, const float *__restrict__ psoft, float *__restrict__ hmx,
-                            float *__restrict__ hmn) {
-    const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (node >= total || t.nchild[node] != 0)
-        return;
-    const uint32_t f = t.first[node], e = f + t.count[node];
-    uint32_t p = node ? t.parent[node] : 0u;  // the climb's first parent
-    uint32_t q = pre2bfs[node];
-    double m = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
-    float hi = 0.0f, lo = INFINITY;  // largest / smallest softening (per-particle softening only)
-    for (uint32_t s = f; s < e; s += 4) {
-        double ms[4], px[4], py[4], pz[4];
-        float hs[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const uint32_t j = min(s + u, e - 1);
-            ms[u] = (double)smass[j];
-            px[u] = spos[3 * j];
-            py[u] = spos[3 * j + 1];
-            pz[u] = spos[3 * j + 2];
-            hs[u] = psoft ? psoft[j] : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            if (s + u < e) {
-                m = __dadd_rn(m, ms[u]);
-                sx = __dadd_rn(sx, __dmul_rn(ms[u], px[u]));
-                sy = __dadd_rn(sy, __dmul_rn(ms[u], py[u]));
-                sz = __dadd_rn(sz, __dmul_rn(ms[u], pz[u]));
-                if (psoft) {
-                    hi = fmaxf(hi, hs[u]);
-                    lo = fminf(lo, hs[u]);
-                }
-            }
-        }
-    }
-    M[q] = m;
-    S[3 * q] = sx;
-    S[3 * q + 1] = sy;
-    S[3 * q + 2] = sz;
-    if (psoft) {
-        hmx[q] = hi;
-        hmn[q] = lo;
-    }
-    uint32_t cur = (uint32_t)node;
-    while (cur != 0) {
-        // links of this step, loaded ahead of the atomic
-        const uint32_t nc = t.nchild[p];
-        const uint32_t c0 = pre2bfs[p + 1];  // first child; the others follow it
-        const uint32_t pq = pre2bfs[p];
-        const uint32_t pp = p ? t.parent[p] : 0u;
-        // release: this node's sums are visible before the parent learns it is
-        // done; acquire: the last child sees all its siblings' sums
-        cuda::atomic_ref<uint32_t, cuda::thread_scope_device> arrive(t.arrive[p]);
-        if (arrive.fetch_add(1u, cuda::memory_order_acq_rel) != nc - 1)
-            return;  // a sibling still works; it will carry on upwards
-        m = sx = sy = sz = 0.0;
-        hi = 0.0f;
-        lo = INFINITY;
-        for (uint32_t c = c0; c < c0 + nc; c++) {
-            m = __dadd_rn(m, __ldcg(&M[c]));
-            sx = __dadd_rn(sx, __ldcg(&S[3 * c]));
-            sy = __dadd_rn(sy, __ldcg(&S[3 * c + 1]));
-            sz = __dadd_rn(sz, __ldcg(&S[3 * c + 2]));
-            if (psoft) {
-                hi = fmaxf(hi, __ldcg(&hmx[c]));
-                lo = fminf(lo, __ldcg(&hmn[c]));
-            }
-        }
-        M[pq] = m;
-        S[3 * pq] = sx;
-        S[3 * pq + 1] = sy;
-        S[3 * pq + 2] = sz;
-        if (psoft) {
-            hmx[pq] = hi;
-            hmn[pq] = lo;
-        }
-        cur = p;
-        p = pp;
-    }
-}
-
-// Inverse of the breadth-first -> pre-order map.
-__global__ void k_invert(const uint32_t *__restrict__ bfs2pre, int64_t total, uint32_t *__restrict__ pre2bfs) {
-    const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (q < total)
-        pre2bfs[bfs2pre[q]] = (uint32_t)q;
-}
-
-struct NodeOut {
-    float4 *cen, *com;
-    int4 *link;
-    uint8_t *level;
-    uint64_t *prefix;
-    float4 *bcen, *bcom;
-    int4 *blink;
-    float4 *spart;
-    float *nsoft, *bsoft;  // per-particle softening only
-};
-
 // Exact centre of node (lvl, pre) relative to x0: (2 i + 1) L0 2^-(lvl + 1)
 // per axis, i the cell index along the axis read off the key prefix; the
 // power of two is built from its bits (exact scaling, lvl <= 21).
@@ -532,15 +375,349 @@ __device__ __forceinline__ NodeGeom node_geom(uint64_t pre, int lvl, double L0) 
     return g;
 }
 
-// K5a: walk tables that do not need the monopoles, written while the monopole
-// pass climbs.  Pre-order: FP32 geometric centre (exact, on the 2^-22 L0 grid)
-// and side, (skip, first particle, count, leaf flag), level and key prefix
-// for export; breadth-first: centre and (first child, child count, first
-// particle, particle count); and every leaf's particles relative to the FP32
-// leaf centre (FP64 difference rounded to FP32) with their masses.
-__global__ void k_tables(NodeArrays t, const uint32_t *__restrict__ pre2bfs, int64_t total,
-                         const double *__restrict__ spos, const float *__restrict__ smass, double x0, double y0,
-                         double z0, double L0, NodeOut o) {
+// FP32 centre, relative to x0, of the level-lvl cell around a key.  With L0 a
+// power of two (open boundaries) the FP32 product of the odd cell index (at
+// most 22 bits) and half the side is exact, so it has the bits of the FP64
+// product rounded to FP32; FP64 instructions are what bounds k_rank.
+__device__ __forceinline__ float3 leaf_centre(uint64_t key, int lvl, double L0) {
+    const uint64_t pre = key >> (3 * (kMaxLevel - lvl));
+    if (((uint64_t)__double_as_longlong(L0) & 0xfffffffffffffull) == 0ull) {
+        const float half = (float)__dmul_rn(L0, __longlong_as_double((long long)(1022 - lvl) << 52));
+        return make_float3((float)(2u * compact3(pre) + 1u) * half, (float)(2u * compact3(pre >> 1) + 1u) * half,
+                           (float)(2u * compact3(pre >> 2) + 1u) * half);
+    }
+    const NodeGeom g = node_geom(pre, lvl, L0);
+    return make_float3((float)g.rx, (float)g.ry, (float)g.rz);
+}
+
+// K3d. Inverse permutation, positions and masses gathered into key order for
+// the sums over leaves, and each particle's walk record: its position relative
+// to the FP32 centre of its leaf (FP64 difference rounded to FP32) and its
+// mass.  The leaf is known from the key and the leaf level, so this runs while
+// the host reads the node count.
+__global__ void k_rank(const uint32_t *__restrict__ perm, int64_t n, const double *__restrict__ pos,
+                       const float *__restrict__ mass, const float *__restrict__ hsoft,
+                       const uint64_t *__restrict__ key, const uint8_t *__restrict__ leaf_level,
+                       const BuildState *__restrict__ st, uint32_t *__restrict__ rank, double *__restrict__ spos,
+                       float *__restrict__ smass, float *__restrict__ psoft, float4 *__restrict__ spart) {
+    int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (s >= n)
+        return;
+    const uint32_t j = perm[s];
+    rank[j] = (uint32_t)s;
+    const double x = pos[3 * (size_t)j], y = pos[3 * (size_t)j + 1], z = pos[3 * (size_t)j + 2];
+    const float m = mass[j];
+    spos[3 * s] = x;
+    spos[3 * s + 1] = y;
+    spos[3 * s + 2] = z;
+    smass[s] = m;
+    if (hsoft)  // per-particle softening, in key order (checked by k_prepare)
+        psoft[s] = hsoft[j];
+    const float3 c = leaf_centre(key[s], leaf_level[s], st->L0);
+    spart[s] = make_float4((float)__dsub_rn(x, __dadd_rn(st->x0[0], (double)c.x)),
+                           (float)__dsub_rn(y, __dadd_rn(st->x0[1], (double)c.y)),
+                           (float)__dsub_rn(z, __dadd_rn(st->x0[2], (double)c.z)), m);
+}
+
+// Pre-order node arrays of the build.
+struct NodeArrays {
+    uint32_t *first, *count, *skip, *nchild;
+    uint8_t *level;
+    uint64_t *prefix;
+};
+
+constexpr int kLevels = kMaxLevel + 1;
+
+// K3c. The nodes, one thread each (a thread per particle with nodes left the
+// first particle's thread, which starts a node on every level, with some 500
+// dependent loads: 51 us at 2^20, 25 us now): the particle a node starts with
+// is found in the scanned node counts, its level counted from that particle's
+// top one, its end by searching the sorted keys; then the skip index (the
+// first node of the particle just past the cell), the key prefix, the parent
+// (the node above with the same first particle, else the cell found by
+// searching downwards) and, by one atomic per node, the parent's child count.
+// The block's nodes per level go to hist[level][block] for the breadth-first
+// order.
+__global__ void __launch_bounds__(kThreads)
+    k_nodes(const uint64_t *__restrict__ key, int64_t n, int64_t total, const uint32_t *__restrict__ base,
+            const uint8_t *__restrict__ top_level, NodeArrays t, uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[kLevels];
+    if (threadIdx.x < kLevels)
+        h[threadIdx.x] = 0u;
+    __syncthreads();
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p < total) {
+        // the last particle whose first node is at or before p
+        int64_t lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (base[mid] <= (uint32_t)p)
+                lo = mid;
+            else
+                hi = mid - 1;
+        }
+        const uint32_t i = (uint32_t)lo, k = (uint32_t)p - base[i];
+        const int l = top_level[i] + (int)k;
+        const int sh = 3 * (kMaxLevel - l);
+        const uint64_t pre = key[i] >> sh;
+        const uint32_t end = search_up(key, i + 1, (uint32_t)n, (pre + 1) << sh);
+        t.first[p] = i;
+        t.count[p] = end - i;
+        t.skip[p] = end < n ? base[end] : (uint32_t)total;
+        t.level[p] = (uint8_t)l;
+        t.prefix[p] = pre;
+        if (l > 0) {
+            uint32_t par = (uint32_t)p - 1;
+            if (k == 0) {
+                const uint32_t f = search_down(key, i, (pre >> 3) << (sh + 3));
+                par = base[f] + (uint32_t)(l - 1 - top_level[f]);
+            }
+            atomicAdd(&t.nchild[par], 1u);
+        }
+        atomicAdd(&h[l], 1u);
+    }
+    __syncthreads();
+    if (threadIdx.x < kLevels)
+        hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
+}
+
+// K3e. Breadth-first order: a stable counting sort of the pre-order by level.
+// place holds, per level and block of K3c, how many nodes come before; within
+// a block the nodes of a level keep their order.
+__global__ void __launch_bounds__(kThreads)
+    k_level_rank(const uint8_t *__restrict__ level, int64_t total, const uint32_t *__restrict__ place,
+                 uint32_t *__restrict__ pre2bfs) {
+    __shared__ uint32_t h[kThreads / 32][kLevels];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < (kThreads / 32) * kLevels; e += kThreads)
+        (&h[0][0])[e] = 0u;
+    __syncthreads();
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int l = p < total ? (int)level[p] : kLevels;
+    const unsigned same = __match_any_sync(0xffffffffu, l);
+    const unsigned before = __popc(same & ((1u << lane) - 1u));
+    if (l < kLevels && before == 0)
+        h[w][l] = (uint32_t)__popc(same);
+    __syncthreads();
+    if (l < kLevels) {
+        uint32_t q = place[(size_t)l * gridDim.x + blockIdx.x] + before;
+        for (int v = 0; v < w; v++)
+            q += h[v][l];
+        pre2bfs[p] = q;
+    }
+}
+
+// K4: FP64 monopoles, bottom-up.  Each leaf sums its particles in sorted
+// order, each node its children in ascending octant order, with explicit
+// round-to-nearest adds / muls, so every sum has the same fixed order and
+// value however the work is divided.  Sums are stored by breadth-first index,
+// where a node's children are contiguous, so that the children's sums load
+// independently.
+//
+// A block takes the nodes that start in a stretch of kStretch sorted particles
+// -- contiguous in the pre-order -- and sums level by level, a block barrier
+// between the levels, the nodes whose subtree ends in the stretch too.  Those
+// that reach past its end all hold the stretch's last particle, so there is
+// one a level at most; they go to late[level][stretch], and k_multipole_late
+// does the same for 32 stretches by one block, again and again until one block
+// has them all.
+//
+// FP64 bounds this (two lanes a cycle and SM, so a warp's FP64 instruction
+// takes the unit 16 cycles however few lanes need it).  Hence the block sorts
+// its leaves by particle count and its nodes by level before it sums: the
+// lanes of a warp have equal work.  (One launch in which the last child of a
+// node to finish, counted with an atomic, sums the node and climbs on: 136 us
+// at 2^20, leaf bucket 16; this without the sort: 100 + 81 with one block for
+// all late nodes; as it is 46 + 28.)
+constexpr int kStretch = 1024;
+constexpr int kLateFan = 32;
+constexpr int kLeafClasses = 17;  // leaves of 1 .. 16 and of more particles
+
+struct Sums {
+    double *v;          // per node mass, mass-weighted x, y, z
+    float *hmx, *hmn;   // largest and smallest support (per-particle softening only)
+};
+
+// Sums the children [c0, c0 + nc) of node q (nc <= 8) in octant order, one of
+// the four components per lane: four lanes share a node's chain of additions.
+__device__ __forceinline__ void sum_children(const Sums &o, uint32_t q, uint32_t c0, uint32_t nc, int comp) {
+    double x[8], sum = 0.0;
+#pragma unroll
+    for (uint32_t u = 0; u < 8; u++)
+        x[u] = __ldcg(&o.v[4 * (size_t)(c0 + min(u, nc - 1)) + comp]);
+#pragma unroll
+    for (uint32_t u = 0; u < 8; u++)
+        if (u < nc)
+            sum = __dadd_rn(sum, x[u]);
+    o.v[4 * (size_t)q + comp] = sum;
+    if (o.hmx && comp < 2) {
+        float *h = comp ? o.hmn : o.hmx;
+        float r = comp ? INFINITY : 0.0f;
+        for (uint32_t c = c0; c < c0 + nc; c++)
+            r = comp ? fminf(r, __ldcg(&h[c])) : fmaxf(r, __ldcg(&h[c]));
+        h[q] = r;
+    }
+}
+
+__global__ void __launch_bounds__(kThreads)
+    k_multipole(NodeArrays t, int64_t n, const uint32_t *__restrict__ base, const uint32_t *__restrict__ pre2bfs,
+                const double *__restrict__ spos, const float *__restrict__ smass, const float *__restrict__ psoft,
+                Sums o, uint32_t *__restrict__ list, uint32_t *__restrict__ late) {
+    constexpr int kClasses = kLeafClasses + kLevels;  // leaves by size, then nodes from the deepest level up
+    __shared__ uint32_t count[kClasses], start[kClasses + 1];
+    const int64_t i0 = (int64_t)blockIdx.x * kStretch, i1 = min(i0 + kStretch, n);
+    const uint32_t p0 = base[i0], p1 = base[i1];
+    if (threadIdx.x < kClasses)
+        count[threadIdx.x] = 0u;
+    if (threadIdx.x < kLevels)
+        late[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = 0xffffffffu;
+    __syncthreads();
+    auto class_of = [&](uint32_t p) {  // -1: late
+        if (t.nchild[p] == 0)
+            return (int)min(t.count[p], (uint32_t)kLeafClasses) - 1;
+        return t.skip[p] > p1 ? -1 : kLeafClasses + kMaxLevel - (int)t.level[p];
+    };
+    for (uint32_t p = p0 + threadIdx.x; p < p1; p += kThreads) {
+        const int c = class_of(p);
+        if (c >= 0)
+            atomicAdd(&count[c], 1u);
+        else
+            late[(size_t)t.level[p] * gridDim.x + blockIdx.x] = p;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t at = p0;
+        for (int c = 0; c < kClasses; c++) {
+            start[c] = at;
+            at += count[c];
+            count[c] = start[c];
+        }
+        start[kClasses] = at;
+    }
+    __syncthreads();
+    for (uint32_t p = p0 + threadIdx.x; p < p1; p += kThreads) {  // any order within a class: each sums by itself
+        const int c = class_of(p);
+        if (c >= 0)
+            list[atomicAdd(&count[c], 1u)] = p;
+    }
+    __syncthreads();
+    for (uint32_t e = start[0] + threadIdx.x; e < start[kLeafClasses]; e += kThreads) {
+        const uint32_t p = list[e];
+        const uint32_t f = t.first[p], end = f + t.count[p], q = pre2bfs[p];
+        double m = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
+        float hi = 0.0f, lo = INFINITY;
+        for (uint32_t s = f; s < end; s += 4) {  // four particles loaded at a time
+            float ms[4], hs[4];
+            double px[4], py[4], pz[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const size_t j = min(s + u, end - 1);
+                ms[u] = smass[j];
+                px[u] = spos[3 * j];
+                py[u] = spos[3 * j + 1];
+                pz[u] = spos[3 * j + 2];
+                hs[u] = psoft ? psoft[j] : 0.0f;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                if (s + u < end) {
+                    const double md = (double)ms[u];
+                    m = __dadd_rn(m, md);
+                    sx = __dadd_rn(sx, __dmul_rn(md, px[u]));
+                    sy = __dadd_rn(sy, __dmul_rn(md, py[u]));
+                    sz = __dadd_rn(sz, __dmul_rn(md, pz[u]));
+                    if (psoft) {
+                        hi = fmaxf(hi, hs[u]);
+                        lo = fminf(lo, hs[u]);
+                    }
+                }
+            }
+        }
+        double2 *v = reinterpret_cast<double2 *>(o.v + 4 * (size_t)q);
+        v[0] = make_double2(m, sx);
+        v[1] = make_double2(sy, sz);
+        if (psoft) {
+            o.hmx[q] = hi;
+            o.hmn[q] = lo;
+        }
+    }
+    for (int c = kLeafClasses; c < kClasses; c++) {
+        if (start[c] == start[c + 1])
+            continue;
+        __syncthreads();
+        for (uint32_t e = start[c] + (threadIdx.x >> 2); e < start[c + 1]; e += kThreads / 4) {
+            const uint32_t p = list[e];
+            sum_children(o, pre2bfs[p], pre2bfs[p + 1], t.nchild[p], threadIdx.x & 3);
+        }
+    }
+}
+
+// The nodes that reach past their stretch: a block per 32 stretches (which
+// together are one stretch of `span` particles), four lanes per stretch, from
+// the deepest level up; those that reach past the block's end go on to out.
+// The links of all levels are loaded first: the chain over the levels is then
+// one load of the children's sums and their additions each.
+__global__ void __launch_bounds__(4 * kLateFan)
+    k_multipole_late(NodeArrays t, int64_t n, const uint32_t *__restrict__ base, const uint32_t *__restrict__ pre2bfs,
+                     Sums o, const uint32_t *__restrict__ late, int64_t stretches, int64_t span,
+                     uint32_t *__restrict__ out) {
+    __shared__ uint32_t node[kLevels][kLateFan], child[kLevels][kLateFan];
+    __shared__ uint8_t number[kLevels][kLateFan];  // of children, 0 for no node
+    __shared__ unsigned levels;
+    const uint32_t end = base[min(((int64_t)blockIdx.x + 1) * span, n)];
+    if (threadIdx.x < kLevels)
+        out[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = 0xffffffffu;
+    if (threadIdx.x == 0)
+        levels = 0u;
+    __syncthreads();
+    for (int e = threadIdx.x; e < kLevels * kLateFan; e += 4 * kLateFan) {
+        const int l = e / kLateFan, u = e % kLateFan;
+        const int64_t b = (int64_t)blockIdx.x * kLateFan + u;
+        const uint32_t p = b < stretches ? late[(size_t)l * stretches + b] : 0xffffffffu;
+        uint32_t nc = 0u;
+        if (p != 0xffffffffu) {
+            if (t.skip[p] > end) {
+                out[(size_t)l * gridDim.x + blockIdx.x] = p;
+            } else {
+                nc = t.nchild[p];
+                node[l][u] = pre2bfs[p];
+                child[l][u] = pre2bfs[p + 1];
+                atomicOr(&levels, 1u << l);
+            }
+        }
+        number[l][u] = (uint8_t)nc;
+    }
+    __syncthreads();
+    const int u = threadIdx.x >> 2, comp = threadIdx.x & 3;
+    for (unsigned todo = levels; todo;) {
+        const int l = 31 - __clz(todo);
+        todo &= ~(1u << l);
+        if (number[l][u])
+            sum_children(o, node[l][u], child[l][u], number[l][u], comp);
+        __syncthreads();
+    }
+}
+
+struct NodeOut {
+    float4 *cen, *com;
+    int4 *link;
+    uint8_t *level;
+    uint64_t *prefix;
+    float4 *bcen, *bcom;
+    int4 *blink;
+    float *nsoft, *bsoft;  // per-particle softening only
+};
+
+// K5: walk tables.  Pre-order: FP32 geometric centre (exact, on the 2^-22 L0
+// grid) and side, centre of mass relative to the exact centre (FP32) and mass,
+// (skip, first particle, count, leaf flag), level and key prefix for export;
+// breadth-first: centre, centre of mass and (first child, child count, first
+// particle, particle count); and the largest softening per node (negative when
+// the node mixes softenings).  S / m is S times the correctly rounded 1 / m:
+// one FP64 reciprocal instead of three divisions; the FP64 product is within
+// an ulp of the quotient, far below the FP32 rounding of the offset.
+__global__ void k_tables(NodeArrays t, const uint32_t *__restrict__ pre2bfs, int64_t total, Sums sums, double x0,
+                         double y0, double z0, double L0, NodeOut o) {
     const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= total)
         return;
@@ -556,37 +733,17 @@ __global__ void k_tables(NodeArrays t, const uint32_t *__restrict__ pre2bfs, int
     o.prefix[p] = pre;
     o.bcen[q] = cen;
     o.blink[q] = make_int4(nch ? (int)pre2bfs[p + 1] : 0, (int)nch, (int)f, (int)c);
-    if (nch == 0) {
-        const double ax = __dadd_rn(x0, (double)cen.x), ay = __dadd_rn(y0, (double)cen.y),
-                     az = __dadd_rn(z0, (double)cen.z);
-        for (uint32_t s = f; s < f + c; s++)
-            o.spart[s] = make_float4((float)__dsub_rn(spos[3 * s], ax), (float)__dsub_rn(spos[3 * s + 1], ay),
-                                     (float)__dsub_rn(spos[3 * s + 2], az), smass[s]);
-    }
-}
-
-// K5b: centre of mass relative to the exact geometric centre (FP32) and mass,
-// pre-order and breadth-first, and the largest softening per node (negative
-// when the node mixes softenings).  S / m is S times the correctly rounded
-// 1 / m: one FP64 reciprocal instead of three divisions; the FP64 product is
-// within an ulp of the quotient, far below the FP32 rounding of the offset.
-__global__ void k_com(NodeArrays t, const uint32_t *__restrict__ pre2bfs, int64_t total,
-                      const double *__restrict__ M, const double *__restrict__ S, const float *__restrict__ hmx,
-                      const float *__restrict__ hmn, double x0, double y0, double z0, double L0, NodeOut o) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= total)
-        return;
-    const uint32_t q = pre2bfs[p];
-    const NodeGeom g = node_geom(t.prefix[p], t.level[p], L0);
-    const double m = M[q];
+    const double2 ms = reinterpret_cast<const double2 *>(sums.v + 4 * (size_t)q)[0],
+                  yz = reinterpret_cast<const double2 *>(sums.v + 4 * (size_t)q)[1];
+    const double m = ms.x;
     const double rm = __drcp_rn(m);
-    const double cx = __dmul_rn(S[3 * q], rm), cy = __dmul_rn(S[3 * q + 1], rm), cz = __dmul_rn(S[3 * q + 2], rm);
+    const double cx = __dmul_rn(ms.y, rm), cy = __dmul_rn(yz.x, rm), cz = __dmul_rn(yz.y, rm);
     const float4 com = make_float4((float)__dsub_rn(cx, __dadd_rn(x0, g.rx)), (float)__dsub_rn(cy, __dadd_rn(y0, g.ry)),
                                    (float)__dsub_rn(cz, __dadd_rn(z0, g.rz)), (float)m);
     o.com[p] = com;
     o.bcom[q] = com;
-    if (hmx) {
-        const float v = hmn[q] < hmx[q] ? -hmx[q] : hmx[q];
+    if (sums.hmx) {
+        const float v = sums.hmn[q] < sums.hmx[q] ? -sums.hmx[q] : sums.hmx[q];
         o.nsoft[p] = v;
         o.bsoft[q] = v;
     }
@@ -665,7 +822,9 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     TPM_CUDA(cudaMemcpyAsync(dst, hst, sizeof(BuildState), cudaMemcpyHostToDevice, st));
 
     // ---- prepare, bounding box and root (last block), keys, sort
-    k_prepare<<<blocks_for(n), kThreads, 0, st>>>(pos_in, mass_in, hsoft_in, n, s->bp.periodic, s->bp.box,
+    // (few blocks, several particles a thread: each block ends in a reduction and
+    // six atomics on the same words)
+    k_prepare<<<std::min(blocks_for(n), (unsigned)(8 * c->num_sms)), kThreads, 0, st>>>(pos_in, mass_in, hsoft_in, n, s->bp.periodic, s->bp.box,
                                                    s->bp.shift[0], s->bp.shift[1], s->bp.shift[2], s->pos, s->mass,
                                                    dst);
     count_launch();
@@ -690,8 +849,9 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     TPM_CUDA(cudaMemcpyAsync(hst, dst, sizeof(BuildState), cudaMemcpyDeviceToHost, st));
     TPM_CUDA(cudaMemcpyAsync(&hst->total, base + n, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     TPM_CUDA(cudaEventRecord(c->ev_state, st));
-    // the particles gathered into key order while the host reads the state
-    k_rank<<<blocks_for(n), kThreads, 0, st>>>(s->perm, n, s->pos, s->mass, hsoft_in, s->rank, spos, smass, s->psoft);
+    // the particles in key order and their walk records while the host reads the state
+    k_rank<<<blocks_for(n), kThreads, 0, st>>>(s->perm, n, s->pos, s->mass, hsoft_in, s->key, leaf_level, dst, s->rank,
+                                               spos, smass, s->psoft, s->spart);
     count_launch();
     TPM_CUDA(cudaGetLastError());
     TPM_CUDA(cudaEventSynchronize(c->ev_state));
@@ -723,36 +883,35 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     // ---- memory for the node passes: scratch in one block, the system's
     // node tables in another
     NodeArrays t{};
-    uint8_t *level_sorted;
-    uint32_t *bfs2pre;
-    float *hmx = nullptr, *hmn = nullptr;
-    size_t lsort_bytes = 0;
-    TPM_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, lsort_bytes, (const uint8_t *)nullptr, (uint8_t *)nullptr,
-                                             (const uint32_t *)nullptr, (uint32_t *)nullptr, (int)nn, 0, 5, st));
-    char *lsort_tmp = cub_tmp;
+    uint32_t *hist, *place, *list, *late, *later;
+    Sums sums{};
+    const unsigned node_blocks = blocks_for(nn);
+    const int64_t cells = (int64_t)kLevels * node_blocks, stretches = (n + kStretch - 1) / kStretch;
+    size_t place_bytes = 0;
+    TPM_CUDA(cub::DeviceScan::ExclusiveSum(nullptr, place_bytes, (const uint32_t *)nullptr, (uint32_t *)nullptr,
+                                           (int)cells, st));
+    char *place_tmp = cub_tmp;
     Carve tmp_b;
-    // nchild and arrive adjacent: one memset clears both
     tmp_b.add(&t.nchild, nn);
-    tmp_b.add(&t.arrive, nn);
     tmp_b.add(&t.first, nn);
     tmp_b.add(&t.count, nn);
     tmp_b.add(&t.skip, nn);
-    tmp_b.add(&t.parent, nn);
-    tmp_b.add(&t.order, nn);
     tmp_b.add(&t.level, nn);
     tmp_b.add(&t.prefix, nn);
-    tmp_b.add(&level_sorted, nn);
-    tmp_b.add(&bfs2pre, nn);
-    if (lsort_bytes > cub_bytes)
-        tmp_b.add(&lsort_tmp, lsort_bytes);
+    tmp_b.add(&hist, cells);
+    tmp_b.add(&place, cells);
+    tmp_b.add(&list, nn);
+    tmp_b.add(&late, kLevels * stretches);
+    tmp_b.add(&later, kLevels * ((stretches + kLateFan - 1) / kLateFan));
+    if (place_bytes > cub_bytes)
+        tmp_b.add(&place_tmp, place_bytes);
     if (s->psoft) {
-        tmp_b.add(&hmx, nn);
-        tmp_b.add(&hmn, nn);
+        tmp_b.add(&sums.hmx, nn);
+        tmp_b.add(&sums.hmn, nn);
     }
     TPM_CHECK(tmp_b.commit(tmp, st));
     Carve sys_b;
-    sys_b.add(&s->msum, nn);  // FP64 sums by breadth-first index, kept with the system for export
-    sys_b.add(&s->ssum, 3 * nn);
+    sys_b.add(&s->msum, 4 * nn);  // FP64 sums by breadth-first index, kept with the system for export
     sys_b.add(&s->pre2bfs, nn);
     sys_b.add(&s->ncen, nn);
     sys_b.add(&s->ncom, nn);
@@ -767,46 +926,34 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
         sys_b.add(&s->bsoft, nn);
     }
     TPM_CHECK(sys_b.commit(s->mem, st));
-    double *M = s->msum, *S = s->ssum;
+    sums.v = s->msum;
     uint32_t *pre2bfs = s->pre2bfs;
 
-    // ---- nodes in pre-order
-    TPM_CUDA(cudaMemsetAsync(t.nchild, 0, (size_t)((char *)t.arrive - (char *)t.nchild) + nn * sizeof(uint32_t), st));
-    k_nodes<<<blocks_for(n), kThreads, 0, st>>>(s->key, n, base, top_level, leaf_level, t);
+    // ---- nodes in pre-order, their breadth-first order, monopoles, tables
+    TPM_CUDA(cudaMemsetAsync(t.nchild, 0, nn * sizeof(uint32_t), st));
+    k_nodes<<<node_blocks, kThreads, 0, st>>>(s->key, n, nn, base, top_level, t, hist);
     count_launch();
     TPM_CUDA(cudaGetLastError());
-
-    // ---- breadth-first order: a stable sort of the pre-order by level
-    TPM_CUDA(cub::DeviceRadixSort::SortPairs(lsort_tmp, lsort_bytes, t.level, level_sorted, t.order, bfs2pre,
-                                             (int)nn, 0, 5, st));
+    TPM_CUDA(cub::DeviceScan::ExclusiveSum(place_tmp, place_bytes, hist, place, (int)cells, st));
     count_cub_call();
-    k_invert<<<blocks_for(nn), kThreads, 0, st>>>(bfs2pre, nn, pre2bfs);
+    k_level_rank<<<node_blocks, kThreads, 0, st>>>(t.level, nn, place, pre2bfs);
     count_launch();
     TPM_CUDA(cudaGetLastError());
-
-    // ---- walk tables and monopoles.  The tables that need no monopole go on
-    // the context's side stream while the monopole pass climbs (its last
-    // levels leave most SMs idle); the centres of mass follow both.
-    NodeOut o{s->ncen, s->ncom,  s->nlink, s->nlevel, s->nprefix, s->bcen,
-              s->bcom, s->blink, s->spart, s->nsoft,  s->bsoft};
-    TPM_CUDA(cudaEventRecord(c->ev_fork, st));
-    TPM_CUDA(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-    k_tables<<<blocks_for(nn), kThreads, 0, c->side>>>(t, pre2bfs, nn, spos, smass, s->x0[0], s->x0[1], s->x0[2],
-                                                       s->L0, o);
-    const cudaError_t e_tab = cudaGetLastError();
-    const cudaError_t e_join = cudaEventRecord(c->ev_join, c->side);
-    k_multipole<<<blocks_for(nn), kThreads, 0, st>>>(t, nn, pre2bfs, spos, smass, M, S, s->psoft, hmx, hmn);
-    const cudaError_t e_mp = cudaGetLastError();
-    // st waits for the side stream before anything (the scratch frees among
-    // them) follows on it; if that cannot be enqueued, the host waits instead
-    const cudaError_t e_wait = e_join == cudaSuccess ? cudaStreamWaitEvent(st, c->ev_join, 0) : e_join;
-    if (e_wait != cudaSuccess)
-        cudaStreamSynchronize(c->side);
-    TPM_CUDA(e_tab);
-    TPM_CUDA(e_wait);
-    TPM_CUDA(e_mp);
-    count_launch(2);
-    k_com<<<blocks_for(nn), kThreads, 0, st>>>(t, pre2bfs, nn, M, S, hmx, hmn, s->x0[0], s->x0[1], s->x0[2], s->L0, o);
+    k_multipole<<<(unsigned)stretches, kThreads, 0, st>>>(t, n, base, pre2bfs, spos, smass, s->psoft, sums, list, late);
+    count_launch();
+    TPM_CUDA(cudaGetLastError());
+    for (int64_t left = stretches, span = (int64_t)kStretch * kLateFan;; span *= kLateFan) {
+        const int64_t blocks = (left + kLateFan - 1) / kLateFan;
+        k_multipole_late<<<(unsigned)blocks, 4 * kLateFan, 0, st>>>(t, n, base, pre2bfs, sums, late, left, span, later);
+        count_launch();
+        TPM_CUDA(cudaGetLastError());
+        if (blocks == 1)
+            break;
+        std::swap(late, later);  // the lists shrink: both have room
+        left = blocks;
+    }
+    NodeOut o{s->ncen, s->ncom, s->nlink, s->nlevel, s->nprefix, s->bcen, s->bcom, s->blink, s->nsoft, s->bsoft};
+    k_tables<<<node_blocks, kThreads, 0, st>>>(t, pre2bfs, nn, sums, s->x0[0], s->x0[1], s->x0[2], s->L0, o);
     count_launch();
     TPM_CUDA(cudaGetLastError());
     return TPM_OK;

@@ -276,20 +276,8 @@ int tpm_create(tpm_ctx **out, int device, size_t budget) {
     cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &thr);
     e = cudaMallocHost(&c->pinned_state, kPinnedStateBytes);
     if (e == cudaSuccess)
-        e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess)
-        e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess)
-        e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess)
         e = cudaEventCreateWithFlags(&c->ev_state, cudaEventDisableTiming);
     if (e != cudaSuccess) {
-        if (c->ev_fork)
-            cudaEventDestroy(c->ev_fork);
-        if (c->ev_join)
-            cudaEventDestroy(c->ev_join);
-        if (c->side)
-            cudaStreamDestroy(c->side);
         if (c->pinned_state)
             cudaFreeHost(c->pinned_state);
         cudaMemPoolDestroy(c->pool);
@@ -325,10 +313,7 @@ int tpm_destroy(tpm_ctx *h) {
     cudaStreamSynchronize(0);
     cudaMemPoolDestroy(c->pool);
     cudaFreeHost(c->pinned_state);
-    cudaEventDestroy(c->ev_fork);
-    cudaEventDestroy(c->ev_join);
     cudaEventDestroy(c->ev_state);
-    cudaStreamDestroy(c->side);
     delete c;
     return TPM_OK;
 }
@@ -751,18 +736,17 @@ int tpm_tree_export(tpm_ctx *h, tpm_sys sid, uint64_t *key, uint32_t *perm, uint
     if (mass || com) {
         // FP64 sums by breadth-first index; the centre of mass is S / m
         // (IEEE division, correctly rounded as on the device)
-        std::vector<double> M(m), S(3 * m);
+        std::vector<double> S(4 * m);
         std::vector<uint32_t> q(m);
-        TPM_CUDA(cudaMemcpy(M.data(), s->msum, m * 8, cudaMemcpyDeviceToHost));
-        TPM_CUDA(cudaMemcpy(S.data(), s->ssum, 3 * m * 8, cudaMemcpyDeviceToHost));
+        TPM_CUDA(cudaMemcpy(S.data(), s->msum, 4 * m * 8, cudaMemcpyDeviceToHost));
         TPM_CUDA(cudaMemcpy(q.data(), s->pre2bfs, m * 4, cudaMemcpyDeviceToHost));
         for (int64_t i = 0; i < m; i++) {
-            const double mi = M[q[i]];
+            const double mi = S[4 * (size_t)q[i]];
             if (mass)
                 mass[i] = mi;
             if (com)
                 for (int a = 0; a < 3; a++)
-                    com[3 * i + a] = S[3 * (size_t)q[i] + a] / mi;
+                    com[3 * i + a] = S[4 * (size_t)q[i] + 1 + a] / mi;
         }
     }
     if (xtree)

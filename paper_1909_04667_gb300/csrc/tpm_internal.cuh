@@ -155,10 +155,9 @@ struct System {
     int4 *blink = nullptr;
     uint8_t *nlevel = nullptr;
     uint64_t *nprefix = nullptr;
-    // FP64 mass and mass-weighted position sums by breadth-first index, and
-    // the pre-order -> breadth-first map (for export)
+    // FP64 sums by breadth-first index, four per node (mass, mass-weighted x,
+    // y, z), and the pre-order -> breadth-first map (for export)
     double *msum = nullptr;
-    double *ssum = nullptr;
     uint32_t *pre2bfs = nullptr;
 
     // device status word: bit 0 an active id was out of range, bit 1 the group
@@ -189,10 +188,6 @@ struct Ctx {
     int device = 0;
     void *pinned_state = nullptr;  // host page for a build's device-side bookkeeping
     std::mutex build_mu;
-    // side stream of the tree build (work that overlaps the monopole pass) and
-    // its fork / join events; used under build_mu
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaEvent_t ev_state = nullptr;  // a build's state has reached the pinned page
     int num_sms = 0;
     size_t budget = 0;
