@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <type_traits>
 
 #include "tpm_internal.cuh"
 
@@ -147,6 +148,93 @@ __device__ __forceinline__ void pair_term_h(float rx, float ry, float rz, float 
     pair_term_s<TREEPM>(rx, ry, rz, r2, m, h2, hinv, hinv3, k, ax, ay, az, ph);
 }
 
+
+// short_range_factors of two distances through the two-wide instructions, each
+// element rounded as there.
+__device__ __forceinline__ void short_range_pair(float2 r, float inv2rs, float2 &gs, float2 &gp) {
+    auto two = [](float v) { return make_float2(v, v); };
+    const float2 u = __fmul2_rn(r, two(inv2rs));
+    const float2 d = __ffma2_rn(two(0.3275911f), u, two(1.0f));
+    const float2 t = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
+    float2 poly = __ffma2_rn(t, two(1.061405429f), two(-1.453152027f));
+    poly = __ffma2_rn(t, poly, two(1.421413741f));
+    poly = __ffma2_rn(t, poly, two(-0.284496736f));
+    poly = __ffma2_rn(t, poly, two(0.254829592f));
+    poly = __fmul2_rn(poly, t);
+    const float2 q = __fmul2_rn(make_float2(-u.x, -u.y), u);
+    const float2 e = make_float2(__expf(q.x), __expf(q.y));
+    gp = __fmul2_rn(poly, e);
+    gs = __ffma2_rn(__fmul2_rn(two(1.1283791671f), u), e, gp);
+}
+
+// Spline-softened force and potential factors at r <= h (Sec. 3.2), both
+// pieces evaluated and one selected.
+__device__ __forceinline__ void spline_factors(float r, float hinv, float hinv3, float &kf, float &kp) {
+    const float u = r * hinv, u2 = u * u;
+    const float iu = __fdividef(1.0f, fmaxf(u, 0.25f));
+    const float f0 = fmaf(u2, fmaf(32.0f, u, -38.4f), 10.666666667f);
+    const float p0 = fmaf(u2, fmaf(u2, fmaf(6.4f, u, -9.6f), 5.333333333f), -2.8f);
+    const float f1 = fmaf(u, fmaf(u, fmaf(-10.666666667f, u, 38.4f), -48.0f), 21.333333333f) -
+                     0.066666666667f * iu * iu * iu;
+    const float p1 = fmaf(u2, fmaf(u, fmaf(u, fmaf(-2.133333333f, u, 9.6f), -16.0f), 10.666666667f), -3.2f) +
+                     0.066666666667f * iu;
+    kf = hinv3 * (u < 0.5f ? f0 : f1);
+    kp = hinv * (u < 0.5f ? p0 : p1);
+}
+
+// Sums of one lane for two targets: sum of m r^-3 (target - source) and of
+// m / r, both with their signs turned when the result is written.
+struct PairSums {
+    float2 x, y, z, p;
+};
+
+// Pair terms of one source with two targets at offset (target - source), for
+// distances beyond the softening length (r2 already raised to h^2), with the
+// short-range factors under TreePM.
+template <bool TREEPM>
+__device__ __forceinline__ void far_pair(float2 rx, float2 ry, float2 rz, float2 r2, float2 m, const WalkConsts &k,
+                                         PairSums &s) {
+    const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+    float2 mr = __fmul2_rn(m, ri);
+    float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
+    if (TREEPM) {
+        float2 gs, gp;
+        short_range_pair(__fmul2_rn(r2, ri), k.inv2rs, gs, gp);
+        mr = __fmul2_rn(mr, gp);
+        mr3 = __fmul2_rn(mr3, gs);
+    }
+    s.x = __ffma2_rn(mr3, rx, s.x);
+    s.y = __ffma2_rn(mr3, ry, s.y);
+    s.z = __ffma2_rn(mr3, rz, s.z);
+    s.p = __fadd2_rn(s.p, mr);
+}
+
+// For a source inside a target's softening length: the difference of the
+// spline term to the term at r = h that far_pair added.
+template <bool TREEPM>
+__device__ __forceinline__ void soft_correction(float rx, float ry, float rz, float r2, float m, float h2, float hinv,
+                                                float hinv3, const WalkConsts &k, float &sx, float &sy, float &sz,
+                                                float &sp) {
+    const float r = sqrtf(r2);
+    float kf, kp;
+    spline_factors(r, hinv, hinv3, kf, kp);
+    const float ri = rsqrtf(h2);
+    float fh = ri * ri * ri, ph = ri;
+    if (TREEPM) {
+        float gs, gp;
+        short_range_factors(r, k.inv2rs, gs, gp);
+        kf *= gs;
+        kp *= gp;
+        short_range_factors(h2 * ri, k.inv2rs, gs, gp);
+        fh *= gs;
+        ph *= gp;
+    }
+    const float f = m * (kf - fh);
+    sx = fmaf(f, rx, sx);
+    sy = fmaf(f, ry, sy);
+    sz = fmaf(f, rz, sz);
+    sp = fmaf(m, -kp - ph, sp);
+}
 
 __device__ __forceinline__ float wrap_min_image(float d, const WalkConsts &k) {
     return fmaf(-k.box, rintf(d * k.boxinv), d);
@@ -1422,6 +1510,7 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
 
 
 #include "walk_few.cuh"
+#include "walk_box.cuh"
 
 // Walks a chunk of consecutive active particles: in one frame, or, when it
 // is spread out (chunk_cuts), run by run, each run in its own frame.
@@ -2105,7 +2194,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 5)
 }
 
 template <bool P, bool R, bool T, bool V>
-void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, int rule, int *err, int num_sms,
+void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, bool box, int rule, int *err, int num_sms,
             cudaStream_t st) {
     const int64_t warps = (r.n_act + 31) / 32;
     if (lanes) {
@@ -2136,6 +2225,14 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
     const size_t smem = kGroupWarps * sizeof(GroupSharedT<kStackCap, V, P>);
     TreeView tv{s->bcen, s->bcom, s->blink, s->spart, s->psoft, s->bsoft, s->key,
                 s->perm, s->pos,  s->x0[0], s->x0[1],  s->x0[2], s->L0};
+    if constexpr (P && T) {
+        if (box) {
+            k_walk_box<R><<<(unsigned)((warps + kBoxWarps - 1) / kBoxWarps), kBoxWarps * 32, 0, st>>>(
+                tv, r.sorted_idx, r.slot, r.a_old, r.n_act, k, r.acc, r.pot, r.nint, err);
+            count_launch();
+            return;
+        }
+    }
     if constexpr (!P) {
         if (rule != kFewNone) {
             const int64_t blocks = (r.n_act + 2 * kFewWarps - 1) / (2 * kFewWarps);
@@ -2162,10 +2259,10 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
 }
 
 // Kernel choice: the group walk for open boundaries (with or without the
-// TreePM split), the lane walk for the periodic short-range walk (there the
-// cutoff sphere, a few mean spacings wide, cuts through most groups, so the
-// group bounds rarely decide and the lane walk is faster).  TPM_WALK=lanes or
-// group forces one for comparison; both make the same per-particle decisions.
+// TreePM split; two targets a warp where few_rule says so), the box walk for
+// the periodic short-range walk, the lane walk for the Ewald tree (its gathers
+// want neighbouring targets in a warp's lanes).  TPM_WALK=lanes or group
+// forces one of those for comparison; all make the same per-particle decisions.
 int walk_override() {
     static int v = -1;
     if (v < 0) {
@@ -2338,7 +2435,8 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
         set_ewald(k, s, tab, phi0);
     }
     const int ov = walk_override();
-    const bool lanes = ov == 1 || (ov == 0 && per);
+    const bool box = ov == 0 && per && tpm;
+    const bool lanes = ov == 1 || (ov == 0 && per && !tpm);
     int *err = s->err;
     if (!per && lanes) {  // the lane walk's list of cut chunks' runs: n_act entries at most
         if (!r.runs || !r.nruns) {
@@ -2359,21 +2457,21 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
             rule = kFewNone;  // all particles: no chunk is sparse
     }
     if (!per && !tpm)
-        rel ? (varh ? launch<false, true, false, true>(s, r, k, lanes, rule, err, c->num_sms, st)
-                    : launch<false, true, false, false>(s, r, k, lanes, rule, err, c->num_sms, st))
-            : (varh ? launch<false, false, false, true>(s, r, k, lanes, rule, err, c->num_sms, st)
-                    : launch<false, false, false, false>(s, r, k, lanes, rule, err, c->num_sms, st));
+        rel ? (varh ? launch<false, true, false, true>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+                    : launch<false, true, false, false>(s, r, k, lanes, box, rule, err, c->num_sms, st))
+            : (varh ? launch<false, false, false, true>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+                    : launch<false, false, false, false>(s, r, k, lanes, box, rule, err, c->num_sms, st));
     else if (!per && tpm)
-        rel ? (varh ? launch<false, true, true, true>(s, r, k, lanes, rule, err, c->num_sms, st)
-                    : launch<false, true, true, false>(s, r, k, lanes, rule, err, c->num_sms, st))
-            : (varh ? launch<false, false, true, true>(s, r, k, lanes, rule, err, c->num_sms, st)
-                    : launch<false, false, true, false>(s, r, k, lanes, rule, err, c->num_sms, st));
+        rel ? (varh ? launch<false, true, true, true>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+                    : launch<false, true, true, false>(s, r, k, lanes, box, rule, err, c->num_sms, st))
+            : (varh ? launch<false, false, true, true>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+                    : launch<false, false, true, false>(s, r, k, lanes, box, rule, err, c->num_sms, st));
     else if (tpm)
-        rel ? launch<true, true, true, false>(s, r, k, lanes, rule, err, c->num_sms, st)
-            : launch<true, false, true, false>(s, r, k, lanes, rule, err, c->num_sms, st);
+        rel ? launch<true, true, true, false>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+            : launch<true, false, true, false>(s, r, k, lanes, box, rule, err, c->num_sms, st);
     else
-        rel ? launch<true, true, false, false>(s, r, k, lanes, rule, err, c->num_sms, st)
-            : launch<true, false, false, false>(s, r, k, lanes, rule, err, c->num_sms, st);
+        rel ? launch<true, true, false, false>(s, r, k, lanes, box, rule, err, c->num_sms, st)
+            : launch<true, false, false, false>(s, r, k, lanes, box, rule, err, c->num_sms, st);
     TPM_CUDA(cudaGetLastError());
     return TPM_OK;
 }

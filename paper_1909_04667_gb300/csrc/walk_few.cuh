@@ -97,76 +97,6 @@ __device__ __forceinline__ RunTargets run_targets(const TreeView &T, const WalkC
     return t;
 }
 
-// Spline-softened force and potential factors at r <= h (Sec. 3.2), both
-// pieces evaluated and one selected.
-__device__ __forceinline__ void spline_factors(float r, float hinv, float hinv3, float &kf, float &kp) {
-    const float u = r * hinv, u2 = u * u;
-    const float iu = __fdividef(1.0f, fmaxf(u, 0.25f));
-    const float f0 = fmaf(u2, fmaf(32.0f, u, -38.4f), 10.666666667f);
-    const float p0 = fmaf(u2, fmaf(u2, fmaf(6.4f, u, -9.6f), 5.333333333f), -2.8f);
-    const float f1 = fmaf(u, fmaf(u, fmaf(-10.666666667f, u, 38.4f), -48.0f), 21.333333333f) -
-                     0.066666666667f * iu * iu * iu;
-    const float p1 = fmaf(u2, fmaf(u, fmaf(u, fmaf(-2.133333333f, u, 9.6f), -16.0f), 10.666666667f), -3.2f) +
-                     0.066666666667f * iu;
-    kf = hinv3 * (u < 0.5f ? f0 : f1);
-    kp = hinv * (u < 0.5f ? p0 : p1);
-}
-
-// Sums of one lane for two targets: sum of m r^-3 (target - source) and of
-// m / r, both with their signs turned when the result is written.
-struct PairSums {
-    float2 x, y, z, p;
-};
-
-// Pair terms of one source with two targets at offset (target - source), for
-// distances beyond the softening length (r2 already raised to h^2), with the
-// short-range factors under TreePM.
-template <bool TREEPM>
-__device__ __forceinline__ void far_pair(float2 rx, float2 ry, float2 rz, float2 r2, float2 m, const WalkConsts &k,
-                                         PairSums &s) {
-    const float2 ri = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
-    float2 mr = __fmul2_rn(m, ri);
-    float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
-    if (TREEPM) {
-        float2 gs, gp;
-        short_range_factors(r2.x * ri.x, k.inv2rs, gs.x, gp.x);
-        short_range_factors(r2.y * ri.y, k.inv2rs, gs.y, gp.y);
-        mr = __fmul2_rn(mr, gp);
-        mr3 = __fmul2_rn(mr3, gs);
-    }
-    s.x = __ffma2_rn(mr3, rx, s.x);
-    s.y = __ffma2_rn(mr3, ry, s.y);
-    s.z = __ffma2_rn(mr3, rz, s.z);
-    s.p = __fadd2_rn(s.p, mr);
-}
-
-// For a source inside a target's softening length: the difference of the
-// spline term to the term at r = h that far_pair added.
-template <bool TREEPM>
-__device__ __forceinline__ void soft_correction(float rx, float ry, float rz, float r2, float m, float h2, float hinv,
-                                                float hinv3, const WalkConsts &k, float &sx, float &sy, float &sz,
-                                                float &sp) {
-    const float r = sqrtf(r2);
-    float kf, kp;
-    spline_factors(r, hinv, hinv3, kf, kp);
-    const float ri = rsqrtf(h2);
-    float fh = ri * ri * ri, ph = ri;
-    if (TREEPM) {
-        float gs, gp;
-        short_range_factors(r, k.inv2rs, gs, gp);
-        kf *= gs;
-        kp *= gp;
-        short_range_factors(h2 * ri, k.inv2rs, gs, gp);
-        fh *= gs;
-        ph *= gp;
-    }
-    const float f = m * (kf - fh);
-    sx = fmaf(f, rx, sx);
-    sy = fmaf(f, ry, sy);
-    sz = fmaf(f, rz, sz);
-    sp = fmaf(m, -kp - ph, sp);
-}
-
 // Exclusive prefix sum over the warp, and the total.
 __device__ __forceinline__ int warp_exclusive(int v, int &total) {
     const int lane = threadIdx.x & 31;
