@@ -375,6 +375,53 @@ __device__ __forceinline__ NodeGeom node_geom(uint64_t pre, int lvl, double L0) 
     return g;
 }
 
+// K2 for small systems: the sorted position of every particle by counting the
+// particles before it, (key, index) below its own, over chunks of kRankChunk
+// others (a block per 256 particles and chunk, the chunk's keys in shared
+// memory).  n^2 comparisons, but two launches: the radix sort takes eight
+// passes of two launches each, some 100 us however few the particles.  A step
+// (build and forces) with the sort / with this: 4096 particles 270 / 190 us,
+// 8192 290 / 222, 16384 340 / 286; the count grows as n^2 (some 45 us at
+// 16384), so the line is drawn at 20480.
+constexpr int64_t kRankSort = 5 << 12;
+constexpr int kRankChunk = 512;
+__global__ void __launch_bounds__(kThreads)
+    k_count_before(const uint64_t *__restrict__ key, int n, uint32_t *__restrict__ rank) {
+    __shared__ __align__(16) uint64_t other[kRankChunk];
+    const int j0 = blockIdx.y * kRankChunk, m = min(kRankChunk, n - j0);
+    for (int e = threadIdx.x; e < kRankChunk; e += kThreads)
+        other[e] = e < m ? key[j0 + e] : ~0ull;  // padding counts for nobody: keys have 63 bits
+    __syncthreads();
+    const int i0 = blockIdx.x * kThreads, i = i0 + threadIdx.x;
+    if (i >= n)
+        return;
+    const uint64_t own = key[i];
+    uint32_t before = 0u;
+    if (j0 + kRankChunk <= i0 || j0 >= i0 + kThreads) {
+        // all of the chunk before this block's particles (equal keys count) or after
+        const uint64_t bound = own + (j0 < i0 ? 1u : 0u);
+        const ulonglong2 *two = reinterpret_cast<const ulonglong2 *>(other);
+#pragma unroll 8
+        for (int e = 0; e < kRankChunk / 2; e++) {
+            const ulonglong2 k = two[e];
+            before += (k.x < bound ? 1u : 0u) + (k.y < bound ? 1u : 0u);
+        }
+    } else {
+        for (int e = 0; e < m; e++)
+            before += other[e] < own + (j0 + e < i ? 1u : 0u) ? 1u : 0u;
+    }
+    atomicAdd(&rank[i], before);
+}
+
+__global__ void k_place(const uint64_t *__restrict__ key, int n, const uint32_t *__restrict__ rank,
+                        uint64_t *__restrict__ sorted, uint32_t *__restrict__ perm) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        sorted[rank[i]] = key[i];
+        perm[rank[i]] = (uint32_t)i;
+    }
+}
+
 // FP32 centre, relative to x0, of the level-lvl cell around a key.  With L0 a
 // power of two (open boundaries) the FP32 product of the odd cell index (at
 // most 22 bits) and half the side is exact, so it has the bits of the FP64
@@ -832,9 +879,17 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     k_keys<<<blocks_for(n), kThreads, 0, st>>>(s->pos, n, dst, key_raw, idx_raw);
     count_launch();
     TPM_CUDA(cudaGetLastError());
-    TPM_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, sort_bytes, key_raw, s->key, idx_raw, s->perm, (int)n, 0,
-                                             3 * kMaxLevel, st));
-    count_cub_call();
+    if (n <= kRankSort) {
+        TPM_CUDA(cudaMemsetAsync(s->rank, 0, n * sizeof(uint32_t), st));
+        k_count_before<<<dim3(blocks_for(n), blocks_for(n, kRankChunk)), kThreads, 0, st>>>(key_raw, (int)n, s->rank);
+        k_place<<<blocks_for(n), kThreads, 0, st>>>(key_raw, (int)n, s->rank, s->key, s->perm);
+        count_launch(2);
+        TPM_CUDA(cudaGetLastError());
+    } else {
+        TPM_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, sort_bytes, key_raw, s->key, idx_raw, s->perm, (int)n, 0,
+                                                 3 * kMaxLevel, st));
+        count_cub_call();
+    }
 
     // ---- node counts per particle and their scan: the pre-order indices
     k_window_max<<<blocks_for((n + B) / ((int64_t)B + 1)), kThreads, 0, st>>>(s->key, n, B, pre_max, suf_max);

@@ -54,6 +54,15 @@ def test_coincident_particles_across_stretches(oracle_mod, ctx):
     check(oracle_mod, ctx, pos, mass, 8)
 
 
+@pytest.mark.parametrize("n", [255, 513, 20480, 20481])
+def test_sorts(oracle_mod, ctx, n):
+    """Both sorts, with equal keys (ties by index) and a last ragged block."""
+    pos, mass = W.plummer(n, n)
+    pos[::7] = pos[3]
+    pos[n // 2:n // 2 + 40] = pos[n - 1]
+    check(oracle_mod, ctx, pos, mass, 4)
+
+
 @pytest.mark.parametrize("scale", [1e-200, 1e-30, 1e30])
 def test_scales(oracle_mod, ctx, scale):
     pos, mass = W.plummer(3000, 5)
