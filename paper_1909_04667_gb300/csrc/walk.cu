@@ -631,7 +631,8 @@ struct GroupSharedT {
     float4 nxy[kNodeCap / 2];
     float4 nzm[kNodeCap / 2];
     uint32_t nmask[kNodeCap];
-    float nsoft[VARH ? kNodeCap : 1];      // its largest spline support (per-particle softening)
+    alignas(8) float nsoft[VARH ? kNodeCap : 2];  // its largest spline support (per-particle softening)
+    float2 psup[VARH ? 16 : 1];            // the particles' supports by pairs
     uint8_t nwrap[PERIODIC ? kNodeCap : 1];
     float4 lsrc[kLeafCap];   // opened leaf: centre (group frame) + first particle
     uint2 lmeta[kLeafCap];   // lane mask, wrap flag | particle count
@@ -767,6 +768,90 @@ __device__ __forceinline__ void newton_term(float rx, float ry, float rz, float 
     ph -= mr;
 }
 
+// Two queued monopoles (paired layout, masses m) for the lane's particle, with
+// the mesh split or per-particle softening; both first at max(r, h).  inside:
+// smallest r^2 - h^2 so far.
+template <bool TREEPM, bool VARH>
+__device__ __forceinline__ void two_nodes(float4 XY, float4 ZM, float2 m, float2 hs, float xox, float xoy, float xoz,
+                                          float hi, const WalkConsts &k, PairSums &s, float &inside) {
+    const float2 rx = __fadd2_rn(make_float2(XY.x, XY.y), make_float2(-xox, -xox));
+    const float2 ry = __fadd2_rn(make_float2(XY.z, XY.w), make_float2(-xoy, -xoy));
+    const float2 rz = __fadd2_rn(make_float2(ZM.x, ZM.y), make_float2(-xoz, -xoz));
+    const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+    float2 h2 = make_float2(k.h2, k.h2);
+    if (VARH) {
+        const float2 he = make_float2(fmaxf(hi, hs.x), fmaxf(hi, hs.y));
+        h2 = __fmul2_rn(he, he);
+    }
+    const float2 d = __ffma2_rn(h2, make_float2(-1.0f, -1.0f), r2);
+    inside = fminf(inside, fminf(d.x, d.y));
+    far_pair<TREEPM>(rx, ry, rz, make_float2(fmaxf(r2.x, h2.x), fmaxf(r2.y, h2.y)), m, k, s);
+}
+
+// Replaces the term at r = h of a source of mass m at offset (rx, ry, rz)
+// inside the support h by its spline term.
+template <bool TREEPM>
+__device__ __forceinline__ void soften_term(float rx, float ry, float rz, float r2, float m, float h,
+                                            const WalkConsts &k, float &ax, float &ay, float &az, float &ph) {
+    const float hi = 1.0f / h;
+    float p = 0.0f;
+    soft_correction<TREEPM>(rx, ry, rz, r2, m, h * h, hi, hi * hi * hi, k, ax, ay, az, p);
+    ph -= p;
+}
+
+// Entries [e0, e1) of the node queue with the mesh split or per-particle
+// softening, two at a time; MASKED: for the lanes in each entry's mask.
+template <bool TREEPM, bool VARH, bool MASKED, class SH>
+__device__ __forceinline__ void sweep_pairs(const SH &sh, int e0, int e1, unsigned lanebit, float xox, float xoy,
+                                            float xoz, float hi, const WalkConsts &k, float &ax, float &ay, float &az,
+                                            float &ph, uint32_t &cnt) {
+    PairSums s;
+    s.x = s.y = s.z = s.p = make_float2(0.f, 0.f);
+    float inside = 1.0f;
+    auto lone = [&](int e, bool mine) {  // an entry without a partner in its pair
+        const float4 A = node_entry(sh, e);
+        const float h = VARH ? sh.nsoft[e] : 0.0f;
+        two_nodes<TREEPM, VARH>(make_float4(A.x, A.x, A.y, A.y), make_float4(A.z, A.z, A.w, A.w),
+                                make_float2(mine ? A.w : 0.0f, 0.0f), make_float2(h, h), xox, xoy, xoz, hi, k, s,
+                                inside);
+    };
+    if (MASKED && (e0 & 1)) {  // the back of the queue ends on a pair, the front starts on one
+        const bool mine = (sh.nmask[e0] & lanebit) != 0u;
+        cnt += mine ? 1u : 0u;
+        lone(e0, mine);
+    }
+    for (int e = (e0 + 1) & ~1; e + 1 < e1; e += 2) {
+        const float4 XY = sh.nxy[e >> 1], ZM = sh.nzm[e >> 1];
+        float2 hs = make_float2(0.f, 0.f), m = make_float2(ZM.z, ZM.w);
+        if (VARH)
+            hs = *reinterpret_cast<const float2 *>(&sh.nsoft[e]);
+        if (MASKED) {
+            const uint2 Mk = *reinterpret_cast<const uint2 *>(&sh.nmask[e]);
+            const bool m0 = (Mk.x & lanebit) != 0u, m1 = (Mk.y & lanebit) != 0u;
+            cnt += (m0 ? 1u : 0u) + (m1 ? 1u : 0u);
+            m = make_float2(m0 ? ZM.z : 0.0f, m1 ? ZM.w : 0.0f);
+        }
+        two_nodes<TREEPM, VARH>(XY, ZM, m, hs, xox, xoy, xoz, hi, k, s, inside);
+    }
+    if (!MASKED && (e1 & 1))
+        lone(e1 - 1, true);
+    ax += s.x.x + s.x.y;
+    ay += s.y.x + s.y.y;
+    az += s.z.x + s.z.y;
+    ph -= s.p.x + s.p.y;
+    if (__any_sync(0xffffffffu, inside < 0.0f)) {
+        const float hk = sqrtf(k.h2);
+        for (int q = e0; q < e1; q++) {
+            const float4 A = node_entry(sh, q);
+            const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
+            const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+            const float h = VARH ? fmaxf(hi, sh.nsoft[q]) : hk;
+            if ((!MASKED || (sh.nmask[q] & lanebit)) && r2 < (VARH ? h * h : k.h2))
+                soften_term<TREEPM>(rx, ry, rz, r2, A.w, h, k, ax, ay, az, ph);
+        }
+    }
+}
+
 // Node entries accepted by every particle of the group sit at the front of the
 // node queue: no lane masks, straight-line Newtonian terms four at a time.
 // With one softening length h every entry first gets the Newtonian term at
@@ -779,7 +864,12 @@ template <bool PERIODIC, bool TREEPM, bool VARH, class SH>
 __device__ __forceinline__ void sweep_full(const SH &sh, int nf, float xox, float xoy, float xoz, float hi,
                                            const WalkConsts &k, float &ax, float &ay, float &az, float &ph,
                                            float4 &ec) {
-    if (TREEPM || PERIODIC) {
+    if (!PERIODIC && (TREEPM || VARH)) {
+        uint32_t none = 0u;
+        sweep_pairs<TREEPM, VARH, false>(sh, 0, nf, 0u, xox, xoy, xoz, hi, k, ax, ay, az, ph, none);
+        return;
+    }
+    if (PERIODIC) {
         for (int e = 0; e < nf; e++) {
             const float4 A = node_entry(sh, e);
             float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
@@ -846,54 +936,6 @@ __device__ __forceinline__ void sweep_full(const SH &sh, int nf, float xox, floa
         }
         return;
     }
-    bool soft = false;
-    int e = 0;
-    for (; e + 3 < nf; e += 4) {
-        float4 A[4];
-#pragma unroll
-        for (int u = 0; u < 4; u++)
-            A[u] = node_entry(sh, e + u);
-#pragma unroll
-        for (int u = 0; u < 4; u++) {
-            const float rx = A[u].x - xox, ry = A[u].y - xoy, rz = A[u].z - xoz;
-            const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            float h2 = k.h2;
-            if (VARH) {
-                const float he = fmaxf(hi, sh.nsoft[e + u]);
-                h2 = he * he;
-            }
-            const bool sf = r2 < h2;
-            soft |= sf;
-            newton_term(rx, ry, rz, sf ? h2 : r2, sf ? 0.0f : A[u].w, ax, ay, az, ph);
-        }
-    }
-    for (; e < nf; e++) {
-        const float4 A = node_entry(sh, e);
-        const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
-        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        float h2 = k.h2;
-        if (VARH) {
-            const float he = fmaxf(hi, sh.nsoft[e]);
-            h2 = he * he;
-        }
-        const bool sf = r2 < h2;
-        soft |= sf;
-        newton_term(rx, ry, rz, sf ? h2 : r2, sf ? 0.0f : A.w, ax, ay, az, ph);
-    }
-    if (__any_sync(0xffffffffu, soft)) {
-        for (int q = 0; q < nf; q++) {
-            const float4 A = node_entry(sh, q);
-            const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
-            const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            if (VARH) {
-                const float he = fmaxf(hi, sh.nsoft[q]);
-                if (r2 < he * he)
-                    pair_term_h<false>(rx, ry, rz, r2, A.w, he, k, ax, ay, az, ph);
-            } else if (r2 < k.h2) {
-                pair_term<false>(rx, ry, rz, r2, A.w, k, ax, ay, az, ph);
-            }
-        }
-    }
 }
 
 // Node entries for a subset of the lanes sit at the back of the node queue
@@ -905,7 +947,11 @@ __device__ __forceinline__ void sweep_partial(const SH &sh, int np, unsigned lan
                                               float xoz, float hi, const WalkConsts &k, float &ax, float &ay,
                                               float &az, float &ph, uint32_t &cnt, float4 &ec) {
     const int e0 = kNodeCap - np;
-    if (TREEPM || PERIODIC) {
+    if (!PERIODIC && (TREEPM || VARH)) {
+        sweep_pairs<TREEPM, VARH, true>(sh, e0, kNodeCap, lanebit, xox, xoy, xoz, hi, k, ax, ay, az, ph, cnt);
+        return;
+    }
+    if (PERIODIC) {
         for (int e = e0; e < kNodeCap; e++) {
             const float4 E = node_entry(sh, e);
             const bool mine = (sh.nmask[e] & lanebit) != 0u;
@@ -978,40 +1024,6 @@ __device__ __forceinline__ void sweep_partial(const SH &sh, int np, unsigned lan
         }
         return;
     }
-    bool soft = false;
-#pragma unroll 2
-    for (int e = e0; e < kNodeCap; e++) {
-        const float4 E = node_entry(sh, e);
-        const bool mine = (sh.nmask[e] & lanebit) != 0u;
-        const float rx = E.x - xox, ry = E.y - xoy, rz = E.z - xoz;
-        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        float h2 = k.h2;
-        if (VARH) {
-            const float he = fmaxf(hi, sh.nsoft[e]);
-            h2 = he * he;
-        }
-        const bool sf = r2 < h2;
-        soft |= mine && sf;
-        const bool use = mine && !sf;
-        cnt += mine ? 1u : 0u;
-        newton_term(rx, ry, rz, use ? r2 : h2, use ? E.w : 0.0f, ax, ay, az, ph);
-    }
-    if (__any_sync(0xffffffffu, soft)) {
-        for (int e = e0; e < kNodeCap; e++) {
-            const float4 E = node_entry(sh, e);
-            const float rx = E.x - xox, ry = E.y - xoy, rz = E.z - xoz;
-            const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            if (!(sh.nmask[e] & lanebit))
-                continue;
-            if (VARH) {
-                const float he = fmaxf(hi, sh.nsoft[e]);
-                if (r2 < he * he)
-                    pair_term_h<false>(rx, ry, rz, r2, E.w, he, k, ax, ay, az, ph);
-            } else if (r2 < k.h2) {
-                pair_term<false>(rx, ry, rz, r2, E.w, k, ax, ay, az, ph);
-            }
-        }
-    }
 }
 
 // Sweeps the queued opened leaves, particle by particle.  With open
@@ -1026,6 +1038,54 @@ __device__ __forceinline__ void sweep_leaves(const SH &sh, int nl, unsigned lane
                                              const float4 *__restrict__ spart, const float *__restrict__ psoft,
                                              const WalkConsts &k, float &ax, float &ay, float &az, float &ph,
                                              uint32_t &cnt, float4 &ec) {
+    if (!PERIODIC && (TREEPM || VARH)) {
+        PairSums s;
+        s.x = s.y = s.z = s.p = make_float2(0.f, 0.f);
+        const float hk = sqrtf(k.h2);
+        for (int e = 0; e < nl; e++) {
+            const float4 E = sh.lsrc[e];
+            const uint2 Mt = sh.lmeta[e];
+            const bool mine = (Mt.x & lanebit) != 0u;
+            // subtract the small particle-to-leaf-centre vector first so that
+            // close pairs keep their precision
+            const float px = xox - E.x, py = xoy - E.y, pz = xoz - E.z;
+            const int j0 = __float_as_int(E.w);
+            const int j1 = j0 + (int)(Mt.y & kLeafCount);
+            for (int jj = j0; jj < j1; jj += 2) {
+                const bool two = jj + 1 < j1;
+                const int jb = two ? jj + 1 : jj;
+                const float4 A = __ldg(&spart[jj]), B = __ldg(&spart[jb]);
+                const float2 qx = __fadd2_rn(make_float2(A.x, B.x), make_float2(-px, -px)),
+                             qy = __fadd2_rn(make_float2(A.y, B.y), make_float2(-py, -py)),
+                             qz = __fadd2_rn(make_float2(A.z, B.z), make_float2(-pz, -pz));
+                const float2 q2 = __ffma2_rn(qx, qx, __ffma2_rn(qy, qy, __fmul2_rn(qz, qz)));
+                float2 he = make_float2(0.f, 0.f), h2 = make_float2(k.h2, k.h2);
+                if (VARH) {
+                    he = make_float2(fmaxf(hi, __ldg(&psoft[jj])), fmaxf(hi, __ldg(&psoft[jb])));
+                    h2 = __fmul2_rn(he, he);
+                }
+                const bool a = mine && (uint32_t)jj != self && (!TREEPM || q2.x <= k.rcut2);
+                const bool b = mine && two && (uint32_t)jb != self && (!TREEPM || q2.y <= k.rcut2);
+                cnt += (a ? 1u : 0u) + (b ? 1u : 0u);
+                far_pair<TREEPM>(qx, qy, qz, make_float2(fmaxf(q2.x, h2.x), fmaxf(q2.y, h2.y)),
+                                 make_float2(a ? A.w : 0.0f, b ? B.w : 0.0f), k, s);
+                // inside a support, at once: with several softening lengths most
+                // leaves near a lane have such a particle
+                const bool ca = a && q2.x < h2.x, cb = b && q2.y < h2.y;
+                if (__any_sync(0xffffffffu, ca || cb)) {
+                    if (ca)
+                        soften_term<TREEPM>(qx.x, qy.x, qz.x, q2.x, A.w, VARH ? he.x : hk, k, ax, ay, az, ph);
+                    if (cb)
+                        soften_term<TREEPM>(qx.y, qy.y, qz.y, q2.y, B.w, VARH ? he.y : hk, k, ax, ay, az, ph);
+                }
+            }
+        }
+        ax += s.x.x + s.x.y;
+        ay += s.y.x + s.y.y;
+        az += s.z.x + s.z.y;
+        ph -= s.p.x + s.p.y;
+        return;
+    }
     if (!TREEPM && !PERIODIC) {
         for (int e = 0; e < nl; e++) {
             const float4 E = sh.lsrc[e];
@@ -1041,32 +1101,19 @@ __device__ __forceinline__ void sweep_leaves(const SH &sh, int nl, unsigned lane
                 const float4 P = __ldg(&spart[jj]);
                 const float qx = P.x - px, qy = P.y - py, qz = P.z - pz;
                 const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-                float h2 = k.h2;
-                if (VARH) {
-                    const float he = fmaxf(hi, __ldg(&psoft[jj]));
-                    h2 = he * he;
-                }
                 const bool use = mine && (uint32_t)jj != self;
-                close |= use && q2 < h2;
+                close |= use && q2 < k.h2;
                 cnt += use ? 1u : 0u;
-                newton_term(qx, qy, qz, fmaxf(q2, h2), use ? P.w : 0.0f, ax, ay, az, ph);
+                newton_term(qx, qy, qz, fmaxf(q2, k.h2), use ? P.w : 0.0f, ax, ay, az, ph);
             }
             if (__any_sync(0xffffffffu, close)) {
                 for (int jj = j0; jj < j1; jj++) {
                     const float4 P = __ldg(&spart[jj]);
                     const float qx = P.x - px, qy = P.y - py, qz = P.z - pz;
                     const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-                    float he = 0.0f, h2 = k.h2;
-                    if (VARH) {
-                        he = fmaxf(hi, __ldg(&psoft[jj]));
-                        h2 = he * he;
-                    }
-                    if (mine && (uint32_t)jj != self && q2 < h2) {
-                        newton_term(qx, qy, qz, h2, -P.w, ax, ay, az, ph);
-                        if (VARH)
-                            pair_term_h<false>(qx, qy, qz, q2, P.w, he, k, ax, ay, az, ph);
-                        else
-                            pair_term<false>(qx, qy, qz, q2, P.w, k, ax, ay, az, ph);
+                    if (mine && (uint32_t)jj != self && q2 < k.h2) {
+                        newton_term(qx, qy, qz, k.h2, -P.w, ax, ay, az, ph);
+                        pair_term<false>(qx, qy, qz, q2, P.w, k, ax, ay, az, ph);
                     }
                 }
             }
@@ -1244,6 +1291,8 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
     float4 ec = make_float4(0.f, 0.f, 0.f, 0.f);  // compensation of the Ewald sums
     uint32_t cnt = 0;
     put_part_entry(sh, lane, make_float4(xox, xoy, xoz, thr));  // read by the transposed decisions
+    if (VARH)
+        reinterpret_cast<float *>(sh.psup)[lane] = hi;
     if (lane == 0) {
         sh.stack[0] = make_uint2(0u, valid_mask);  // the root, breadth-first index 0
         sh.scount[0] = 1;
@@ -1287,7 +1336,7 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
             const float q = RELATIVE ? O.w * L * L : L * L;
             const float gl = 0.6f * L;
             unsigned om = 0u, am = 0u;
-            if (!PERIODIC && !TREEPM && !VARH) {
+            if (!PERIODIC) {
                 // particle pairs through the two-wide FP32 instructions; each
                 // element is rounded as in the scalar form, so the decisions
                 // are the same bits
@@ -1295,6 +1344,7 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
                 const float2 ox = make_float2(O.x, O.x), oy = make_float2(O.y, O.y), oz = make_float2(O.z, O.z);
                 const float2 m1 = make_float2(-1.0f, -1.0f);
                 const bool guard_on = k.box_guard != 0;
+                const float mixed2 = VARH && hsig < 0.0f ? hsig * hsig : 0.0f;  // of a node of mixed softenings
                 unsigned uy = U.y;  // lane bits still to decide, particle pair i in bits 0-1
 #pragma unroll 2
                 for (int i = 0; i < 16; i++, uy >>= 2) {
@@ -1309,11 +1359,26 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
                         t = __fmul2_rn(t, r2);
                     const bool g0 = guard_on && fmaxf(fabsf(px.x), fmaxf(fabsf(py.x), fabsf(pz.x))) <= gl;
                     const bool g1 = guard_on && fmaxf(fabsf(px.y), fmaxf(fabsf(py.y), fabsf(pz.y))) <= gl;
-                    const bool o0 = g0 || q > t.x, o1 = g1 || q > t.y;
+                    bool o0 = g0 || q > t.x, o1 = g1 || q > t.y;
+                    if (VARH) {  // Sec. 3.2: a node of mixed softenings is opened inside its largest one
+                        const float2 hp = sh.psup[i];
+                        o0 = o0 || (hp.x < -hsig && r2.x < mixed2);
+                        o1 = o1 || (hp.y < -hsig && r2.y < mixed2);
+                    }
+                    bool n0 = uy & 1u, n1 = uy & 2u;
+                    if (TREEPM) {  // neither opened nor accepted beyond the cutoff
+                        const float hl = 0.5f * L;
+                        float ex = fmaxf(fabsf(px.x) - hl, 0.0f), ey = fmaxf(fabsf(py.x) - hl, 0.0f),
+                              ez = fmaxf(fabsf(pz.x) - hl, 0.0f);
+                        n0 = n0 && !(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > k.rcut2);
+                        ex = fmaxf(fabsf(px.y) - hl, 0.0f), ey = fmaxf(fabsf(py.y) - hl, 0.0f),
+                        ez = fmaxf(fabsf(pz.y) - hl, 0.0f);
+                        n1 = n1 && !(fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > k.rcut2);
+                    }
                     const unsigned b0 = 1u << (2 * i), b1 = 2u << (2 * i);
-                    if (uy & 1u)
+                    if (n0)
                         o0 ? (om |= b0) : (am |= b0);
-                    if (uy & 2u)
+                    if (n1)
                         o1 ? (om |= b1) : (am |= b1);
                 }
             } else {
@@ -1387,13 +1452,10 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
             const int ntake = take ? min(c, cap - excl) : 0;
             const int nwhole = __popc(__ballot_sync(FULL, whole));
             const int ncand = min(__shfl_sync(FULL, incl, 31), cap);
-            // candidate `lane` comes from the range r whose prefix sums
-            // bracket it (binary search over the nondecreasing incl)
-            int r = 0;
-#pragma unroll
-            for (int b = 16; b > 0; b >>= 1)
-                if (__shfl_sync(FULL, incl, r + b - 1) <= lane)
-                    r += b;
+            // candidate `lane` comes from the last range that starts at or
+            // before it: a bit per range at its first candidate
+            const unsigned starts = __reduce_or_sync(FULL, take ? 1u << excl : 0u);
+            const int r = __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
             const uint32_t cnode = __shfl_sync(FULL, R.x, r) + (uint32_t)(lane - __shfl_sync(FULL, excl, r));
             const uint32_t cmask = __shfl_sync(FULL, R.y, r);
             if (take && !whole) {  // the partly taken range stays on top
@@ -1537,9 +1599,11 @@ __device__ __forceinline__ void walk_runs_of_chunk(const TreeView &T, const Walk
 
 // One warp per group of 32 consecutive active particles.  Seven blocks
 // of four warps per SM: the register cap (72) that keeps the paired FP32
-// sweeps and decisions free of spills (measured against caps of 64 and none).
+// sweeps and decisions free of spills (measured against caps of 64 and none);
+// six with the mesh split (500009 particles and mesh, 7 / 6 blocks: 2.00 /
+// 1.92 ms a step).
 template <bool PERIODIC, bool RELATIVE, bool TREEPM, bool VARH>
-__global__ void __launch_bounds__(kGroupWarps * 32, 7)
+__global__ void __launch_bounds__(kGroupWarps * 32, TREEPM ? 6 : 7)
     k_walk_group(TreeView T, const uint32_t *__restrict__ sidx, const uint32_t *__restrict__ slot,
                  const float *__restrict__ a_old, int64_t n_act, int rule, WalkConsts k, float *__restrict__ acc,
                  float *__restrict__ pot, uint32_t *__restrict__ nint, int accumulate, int *__restrict__ err) {
@@ -1803,11 +1867,8 @@ __device__ __forceinline__ void group_walk64(const TreeView &T, const WalkConsts
                 const int ntake = take ? min(c, cap - excl) : 0;
                 const int nwhole = __popc(__ballot_sync(FULL, whole));
                 const int ncand = min(__shfl_sync(FULL, incl, 31), cap);
-                int r = 0;
-#pragma unroll
-                for (int b = 16; b > 0; b >>= 1)
-                    if (__shfl_sync(FULL, incl, r + b - 1) <= lane)
-                        r += b;
+                const unsigned starts = __reduce_or_sync(FULL, take ? 1u << excl : 0u);
+                const int r = __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
                 const uint32_t cnode = __shfl_sync(FULL, rchild, r) + (uint32_t)(lane - __shfl_sync(FULL, excl, r));
                 const unsigned long long cmask = __shfl_sync(FULL, rmask, r);
                 if (take && !whole) {  // the partly taken range stays on top
