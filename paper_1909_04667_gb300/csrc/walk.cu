@@ -23,6 +23,7 @@
 // a sum of small, accurately rounded terms and the pair arithmetic runs in
 // FP32 with FP32 accumulation.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
@@ -2288,8 +2289,17 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
                 s->perm, s->pos,  s->x0[0], s->x0[1],  s->x0[2], s->L0};
     if constexpr (P && T) {
         if (box) {
-            k_walk_box<R><<<(unsigned)((warps + kBoxWarps - 1) / kBoxWarps), kBoxWarps * 32, 0, st>>>(
-                tv, r.sorted_idx, r.slot, r.a_old, r.n_act, k, r.acc, r.pot, r.nint, err);
+            // warps per chunk: four while they fit the chip about once, two up
+            // to twice (steps with 1 / 2 / 4: 40^3 0.98 / 0.82 / 0.78 ms, 52^3
+            // 0.84 / 0.82 / 0.85, 64^3 2.16 / 2.07 / 2.04, 80^3 2.61 / 2.66 / 2.82)
+            const int split = warps <= 24 * (int64_t)num_sms ? 4 : warps <= 64 * (int64_t)num_sms ? 2 : 1;
+            // cell sides are the box halved: the largest not above the cutoff
+            int level = 0;
+            while (ldexp(s->L0, -level) > std::sqrt((double)k.rcut2) && level < kMaxLevel)
+                level++;
+            k_walk_box<R><<<(unsigned)((warps * split + kBoxWarps - 1) / kBoxWarps), kBoxWarps * 32, 0, st>>>(
+                tv, r.sorted_idx, r.slot, r.a_old, r.n_act, split, (float)ldexp(s->L0, -level), k, r.acc, r.pot, r.nint,
+                err);
             count_launch();
             return;
         }

@@ -2,7 +2,8 @@
 oracle TreePM: few particles in large leaves, a ragged last group, sparse
 targets (groups wider than an eighth of the box, whose nodes have different
 images for different targets), leaves of more than 32 particles, boxes that are
-no power of two, particles clustered across the box's corner.  Identical counts
+no power of two, particles clustered across the box's corner, and four and two
+warps per group (one: the full-size box of test_gpu_fullsize).  Identical counts
 up to FP32 margin flips; forces within 1e-4 (p99) and 1e-3 (max) of the rms
 force, the tolerance of the FP32 mesh."""
 import numpy as np
@@ -21,7 +22,7 @@ def dev(x):
 
 CASES = [("uniform", 40, 40, 1.0, 32, 8), ("uniform", 3001, 3001, 0.7, 32, 8), ("uniform", 3001, 50, 1.0, 32, 64),
          ("uniform", 20000, 20000, 2.5, 64, 4), ("uniform", 20000, 33, 2.5, 64, 1), ("corner", 2500, 2500, 1.0, 64, 48),
-         ("one", 1000, 1, 3.0, 32, 8)]
+         ("one", 1000, 1, 3.0, 32, 8), ("uniform", 150000, 150000, 1.0, 64, 8)]
 
 
 @pytest.mark.parametrize("crit", ["bh", "rel"])
