@@ -15,9 +15,10 @@
 // those in reach taken two at a time through the two-wide instructions.
 // Bound by instruction issue (57 thousand warp instructions for 32 targets, the
 // lane walk 71 thousand): 128^3 box, relative criterion, 4.68 -> 3.7 ms; 40^3
-// box, theta = 0.5, 0.59 -> 0.53 ms.  Images looked up per node instead of per
-// target where one serves the whole group: 6.15 -> 5.4 ms a step.
-
+// box, theta = 0.5, 0.59 -> 0.53 ms; a Zel'dovich box of 128^3 with 98
+// interactions a particle, cold caches, 5.18 -> 4.67 ms (65 thousand
+// instructions).  Images looked up per node instead of per target where one
+// serves the whole group: 6.15 -> 5.4 ms a step.
 //
 // Small boxes leave the chip idle behind 32-target warps (40^3: 2000 of them,
 // four to six thousand fit).  Then `split` warps of a block share a chunk: all

@@ -18,8 +18,8 @@
 // Measured, one force call on the relative criterion (Hernquist, leaf bucket
 // 16), group walk / this walk: 1000 random particles of 2^20 1.24 / 0.07 ms,
 // 16384 of 2^20 0.86 / 0.15 ms, 65536 of 2^20 0.72 / 0.34 ms, 32768 of 2^17
-// 0.43 / 0.19 ms; tree build and forces on a whole small system: 4096 0.42 /
-// 0.30 ms, 32768 0.59 / 0.45 ms; all of 2^20 1.58 / 3.8 ms.  One target a warp
+// 0.43 / 0.19 ms; tree build and forces on a whole small system: 4096 0.32 /
+// 0.20 ms, 32768 0.52 / 0.42 ms; all of 2^20 1.58 / 3.8 ms.  One target a warp
 // or four took 63 and 95 us for the 1000, 547 and 346 us for the 65536.
 
 // A run's targets as one warp's registers: lane l holds target l.
