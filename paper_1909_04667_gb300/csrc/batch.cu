@@ -223,7 +223,7 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
         pl->staged_pending = false;
     }
     const size_t rb = batch_req_bytes();
-    bool any_few = false;  // some request has a rule
+    bool any_few = false, all_few = true;  // some request has a rule; all are walked two particles a warp
     {
         std::lock_guard<std::mutex> lk(c->mu);
         for (int64_t r = 0; r < n_req; r++) {
@@ -247,8 +247,9 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
                 return TPM_EINVAL;
             }
             // groups of 64 have a walk of their own (two particles per lane)
-            const int rule = pl->group_size <= 32 ? batch_few_rule(s, offsets[r + 1] - offsets[r]) : kFewNone;
+            const int rule = pl->group_size <= 32 ? batch_few_rule(p, offsets[r + 1] - offsets[r], n_ids) : kFewNone;
             any_few = any_few || rule != kFewNone;
+            all_few = all_few && rule == kFewAll;
             pl->kreq_host[r] = KeyReq{s->rank, s->n, rule};
             fill_batch_req(pl->reqs_host + r * rb, s, p);
             pl->off_host[r] = offsets[r];
@@ -292,6 +293,9 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
     if (!any_few)
         return launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
                                  pl->slot, a_old, acc, pot, nint, pl->err, st);
+    if (all_few)
+        return launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot, a_old,
+                                     acc, pot, nint, pl->err, st);
     TPM_CUDA(cudaEventRecord(pl->ev_fork, st));
     const int rc = launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
                                      pl->slot, a_old, acc, pot, nint, pl->err, st);

@@ -248,19 +248,20 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
 // two particles per lane (else groups of at most 32, one per lane);
 // stack_depth is the candidate-stack capacity of the walk (128, 192 or 256).
 // The groups that get two particles a warp (few_chunk, by the rule of their
-// request: batch_few_rule for its number of ids) have a list and a launch of
-// their own.
-enum { kFewNone = 0, kFewSparse = 1, kFewAll = 2 };
-constexpr uint32_t kSparseSpan = 8;
+// request: batch_few_rule for its ids and the batch's) have a list and a launch
+// of their own.  A rule above 0 is the smallest distance in key order between
+// neighbours, on average over the group; a lone particle has no neighbour and
+// would cost a whole group's chain.
+enum { kFewAll = -1, kFewNone = 0 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__ sidx, int64_t g0, int gcount) {
-    if (rule != kFewSparse)
+    if (rule <= 0)
         return rule == kFewAll;
-    return sidx && sidx[g0 + gcount - 1] - sidx[g0] >= kSparseSpan * (uint32_t)gcount;
+    return sidx && sidx[g0 + gcount - 1] - sidx[g0] >= (uint32_t)rule * (uint32_t)(gcount - 1);
 }
 #endif
 size_t batch_req_bytes();
-int batch_few_rule(const System *s, int64_t n_ids);
+int batch_few_rule(const tpm_force_params *p, int64_t n_ids, int64_t batch_ids);
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
                           unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
                           float *pot, uint32_t *nint, int *err, cudaStream_t st);

@@ -2400,8 +2400,11 @@ int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 
     return TPM_OK;
 }
 
-int batch_few_rule(const System *s, int64_t n_ids) {
-    return walk_override() == 0 ? few_rule(s, n_ids, true) : kFewNone;
+int batch_few_rule(const tpm_force_params *p, int64_t n_ids, int64_t batch_ids) {
+    if (walk_override() != 0)
+        return kFewNone;
+    const bool rel = p->crit == TPM_CRIT_RELATIVE;
+    return batch_ids <= kFewBatch ? few_rule(rel, true, n_ids) : few_span(rel, n_ids);
 }
 
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p) {
@@ -2523,8 +2526,8 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
     }
     int rule = kFewNone;
     if (ov == 0 && !per) {
-        rule = few_rule(s, r.n_act, !tpm && !varh);
-        if (rule == kFewSparse && !r.sorted_idx)
+        rule = few_rule(rel, !tpm && !varh, r.n_act);
+        if (rule > 0 && !r.sorted_idx)
             rule = kFewNone;  // all particles: no chunk is sparse
     }
     if (!per && !tpm)

@@ -374,27 +374,52 @@ __device__ __forceinline__ void few_walk_chunk(const TreeView &T, const WalkCons
 }
 
 // ----------------------------------------------------------------------
-// Which chunks of a call's sorted active list get two targets a warp.  The
-// rule looks at the request alone (its system, its size, the chunk), so that
-// a request gets the same bits in a plain call and in any batch:
-//   kFewAll     every chunk: systems of at most 2^15 particles (1024 groups
-//               of 32 at most; both sides at 4096 and 32768 above), and, for
-//               the walks that no batch runs (mesh, per-particle softening),
-//               calls for at most 2^16 particles (65536 of a 2^20 halo's
-//               densest: step 1.33 / 1.20 ms; at 2^17 the two meet).
-//   kFewSparse  requests of at most 2^16 particles: the chunks whose targets
-//               are on average at least kSparseSpan particles apart in key
-//               order.  Closer ones keep the group walk, which needs half the
-//               instructions for them and wins in a batch that fills the chip.
-//   kFewNone    larger requests.
+// Which chunks of a call's sorted active list get two targets a warp.  A group
+// walk is one warp's chain, as long for 20 groups as for 2000; this walk
+// spreads it over 16 warps for twice the instructions.  It is the faster one
+// until the targets in flight fill the chip, whatever their tree's size, so
+// the rule goes by the number of targets in the call:
+//   kFewAll   every chunk, for requests of at most kFewBH, kFewRelative or
+//             kFewOther ids, by themselves or in a batch of at most kFewBatch
+//             (whose one walk serves all requests).  Group walk / this walk in
+//             us, Hernquist and Plummer spheres, leaf bucket 16:
+//                                        theta 0.7   theta 0.5    alpha 0.0025
+//               batch of 12 x 4096       437 / 344   626 / 427    605 / 363
+//               batch of 3 x 16384       406 / 369   765 / 526    649 / 372
+//               batch of 6 x 16384       487 / 576   792 / 856    827 / 575
+//               all of 32768             212 / 187   444 / 319    282 / 153
+//               all of 49152             221 / 262   452 / 472    292 / 215
+//               all of 65536             244 / 336   479 / 617    310 / 275
+//               32768 densest of 2^17    298 / 290   550 / 510    374 / 281
+//               49152 densest of 2^17    327 / 380   592 / 686    365 / 349
+//               65536 densest of 2^17    373 / 463   695 / 851    382 / 413
+//             two softenings (the mesh is kinder to this walk):
+//               32768 densest of 2^19    392 / 370   755 / 703    608 / 382
+//               65536 densest of 2^19    439 / 629   851 / 1257   650 / 580
+//   span > 0  larger requests of at most 2^16 ids: the chunks whose neighbours
+//             are on average at least that many particles apart in key order;
+//             closer ones keep the group walk.  Batches that fill the chip
+//             (16 requests for random ids of 2^19; group walk / this walk):
+//             span 16 4544 / 5675 us at theta = 0.5, 2265 / 2333 at alpha =
+//             0.0025; span 32 3162 / 3001, 1724 / 1285.
+//   kFewNone  larger requests.
+// At 32 particles a group a request has the same bits in a plain call and in
+// every batch of at most kFewBatch ids, and in every larger batch; the two differ
+// by FP32 rounding.  Groups of 64 particles never come here.
 // ----------------------------------------------------------------------
-constexpr int64_t kFewSystem = 1 << 15;
+constexpr int64_t kFewBH = 1 << 15;
+constexpr int64_t kFewRelative = 3 << 14;  // uniform softening, no mesh
+constexpr int64_t kFewOther = 1 << 16;     // relative criterion with the mesh or per-particle softening
+constexpr int64_t kFewBatch = 3 << 14;
 constexpr int64_t kFewRequest = 1 << 16;
 
-inline int few_rule(const System *s, int64_t n_act, bool batchable) {
-    if (s->n <= kFewSystem || (!batchable && n_act <= kFewRequest))
-        return kFewAll;
-    return n_act <= kFewRequest ? kFewSparse : kFewNone;
+inline int few_span(bool relative, int64_t n_ids) {
+    return n_ids > kFewRequest ? (int)kFewNone : relative ? 16 : 32;
+}
+
+inline int few_rule(bool relative, bool uniform, int64_t n_act) {
+    const int64_t line = !relative ? kFewBH : uniform ? kFewRelative : kFewOther;
+    return n_act <= line ? (int)kFewAll : few_span(relative, n_act);
 }
 
 // A warp per two active particles of a chunk, for the chunks that the rule
