@@ -15,8 +15,8 @@
 //      (G is the plan's group size, chosen by tpm_plan_autotune); those that
 //      get two particles a warp (small or sparse requests) are listed apart,
 //   3. one persistent walk launch lets resident warps take groups from a
-//      device work queue until it is empty, and another does the same for the
-//      groups listed apart, two particles an item.
+//      device work queue until it is empty, and another, beside it in the same
+//      stream, does so for the groups listed apart, two particles an item.
 #include <cub/cub.cuh>
 
 #include <algorithm>
@@ -58,10 +58,6 @@ struct Plan {
     size_t cub_bytes = 0;
     cudaEvent_t staged = nullptr;  // host staging buffers may be rewritten once this has passed
     bool staged_pending = false;
-    // the groups that get two particles a warp are walked on a stream of the
-    // plan's own, beside the others: they fill the tail of that launch
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
 };
 
 // Per requested id (one thread each, over all requests: one block per
@@ -172,14 +168,6 @@ void release_plan(Plan *pl) {
         cudaFreeHost(pl->reqs_host);
     if (pl->staged)
         cudaEventDestroy(pl->staged);
-    if (pl->ev_fork)
-        cudaEventDestroy(pl->ev_fork);
-    if (pl->ev_join)
-        cudaEventDestroy(pl->ev_join);
-    if (pl->side)
-        cudaStreamDestroy(pl->side);
-    pl->ev_fork = pl->ev_join = nullptr;
-    pl->side = nullptr;
     pl->off_host = nullptr;
     pl->kreq_host = nullptr;
     pl->reqs_host = nullptr;
@@ -290,22 +278,13 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
                                                     pl->groups, pl->ngroups, pl->few, pl->nfew);
     count_launch();
     TPM_CUDA(cudaGetLastError());
-    if (!any_few)
-        return launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
-                                 pl->slot, a_old, acc, pot, nint, pl->err, st);
-    if (all_few)
-        return launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot, a_old,
-                                     acc, pot, nint, pl->err, st);
-    TPM_CUDA(cudaEventRecord(pl->ev_fork, st));
-    const int rc = launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
-                                     pl->slot, a_old, acc, pot, nint, pl->err, st);
-    TPM_CUDA(cudaStreamWaitEvent(pl->side, pl->ev_fork, 0));
-    const int rc_few = launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot,
-                                             a_old, acc, pot, nint, pl->err, pl->side);
-    // the caller's stream goes on when both are done, whatever the launches said
-    TPM_CUDA(cudaEventRecord(pl->ev_join, pl->side));
-    TPM_CUDA(cudaStreamWaitEvent(st, pl->ev_join, 0));
-    return rc != TPM_OK ? rc : rc_few;
+    if (!all_few)
+        TPM_CHECK(launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
+                                    pl->slot, a_old, acc, pot, nint, pl->err, st));
+    if (any_few)
+        TPM_CHECK(launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot,
+                                        a_old, acc, pot, nint, pl->err, !all_few, st));
+    return TPM_OK;
 }
 
 }  // namespace
@@ -368,10 +347,7 @@ int tpm_plan_create(tpm_ctx *h, int64_t max_ids, int64_t max_requests, tpm_plan 
     if (cudaMallocHost(&pl->off_host, (max_requests + 1) * sizeof(int64_t)) != cudaSuccess ||
         cudaMallocHost(&pl->kreq_host, max_requests * sizeof(KeyReq)) != cudaSuccess ||
         cudaMallocHost(&pl->reqs_host, max_requests * rb) != cudaSuccess ||
-        cudaEventCreateWithFlags(&pl->staged, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&pl->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&pl->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&pl->side, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaEventCreateWithFlags(&pl->staged, cudaEventDisableTiming) != cudaSuccess) {
         set_error("pinned staging allocation failed");
         return fail(TPM_ECUDA);
     }

@@ -251,7 +251,8 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
 // request: batch_few_rule for its ids and the batch's) have a list and a launch
 // of their own.  A rule above 0 is the smallest distance in key order between
 // neighbours, on average over the group; a lone particle has no neighbour and
-// would cost a whole group's chain.
+// would cost a whole group's chain.  beside: the launch directly follows
+// launch_walk_batch's in the stream and may overlap it.
 enum { kFewAll = -1, kFewNone = 0 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__ sidx, int64_t g0, int gcount) {
@@ -264,7 +265,7 @@ size_t batch_req_bytes();
 int batch_few_rule(const tpm_force_params *p, int64_t n_ids, int64_t batch_ids);
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
                           unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
-                          float *pot, uint32_t *nint, int *err, cudaStream_t st);
+                          float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st);
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p);
 int launch_walk_batch(Ctx *c, int group_size, int stack_depth, const void *reqs, const uint4 *groups,
                       const unsigned *n_groups, unsigned *next, const uint32_t *sidx, const uint32_t *slot,

@@ -1611,6 +1611,8 @@ __global__ void __launch_bounds__(kGroupWarps * 32, TREEPM ? 6 : 7)
     using SH = GroupSharedT<kStackCap, VARH, PERIODIC>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SH &sh = reinterpret_cast<SH *>(smem_raw)[threadIdx.x >> 5];
+    if (!PERIODIC && rule > 0)
+        cudaTriggerProgrammaticLaunchCompletion();  // the other chunks' walk may start beside this one
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t g0 = warp * 32;
     if (g0 >= n_act)
@@ -2147,6 +2149,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 7)
     BatchReq &R = breq[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
     const unsigned total = *n_groups;
+    cudaTriggerProgrammaticLaunchCompletion();  // the two-target walk may start beside this one
     for (;;) {
         unsigned g = 0;
         if (lane == 0)
@@ -2213,6 +2216,7 @@ __global__ void __launch_bounds__(kFewWarps * 32)
                                                 0, err);
         __syncwarp();
     }
+    end_after_group_walk();
 }
 
 // The persistent batch walk with 64-particle groups (open boundaries, one
@@ -2304,14 +2308,13 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
             return;
         }
     }
+    const unsigned few_blocks = (unsigned)((r.n_act + 2 * kFewWarps - 1) / (2 * kFewWarps));
     if constexpr (!P) {
-        if (rule != kFewNone) {
-            const int64_t blocks = (r.n_act + 2 * kFewWarps - 1) / (2 * kFewWarps);
-            k_walk_few<R, T, V><<<(unsigned)blocks, kFewWarps * 32, 0, st>>>(
+        if (rule == kFewAll) {
+            k_walk_few<R, T, V><<<few_blocks, kFewWarps * 32, 0, st>>>(
                 tv, r.sorted_idx, r.slot, r.a_old, r.n_act, rule, k, r.acc, r.pot, r.nint, r.accumulate, err);
             count_launch();
-            if (rule == kFewAll)
-                return;
+            return;
         }
     }
     if (!lanes) {
@@ -2319,6 +2322,15 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
         k_walk_group<P, R, T, V><<<(unsigned)blocks, kGroupWarps * 32, smem, st>>>(
             tv, r.sorted_idx, r.slot, r.a_old, r.n_act, rule, k, r.acc, r.pot, r.nint, r.accumulate, err);
         count_launch();
+        if constexpr (!P) {
+            if (rule > 0) {
+                cudaLaunchAttribute attr;
+                const cudaLaunchConfig_t cfg = beside_config(few_blocks, kFewWarps * 32, &attr, st);
+                cudaLaunchKernelEx(&cfg, k_walk_few<R, T, V>, tv, r.sorted_idx, r.slot, r.a_old, r.n_act, rule, k,
+                                   r.acc, r.pot, r.nint, r.accumulate, err);
+                count_launch();
+            }
+        }
     } else if constexpr (!P) {
         // the lane walk hands spread-out chunks to the group walk: their runs
         // (rare: usually none, and the launch returns at once)
@@ -2383,7 +2395,7 @@ size_t batch_req_bytes() { return sizeof(BatchReq); }
 
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
                           unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
-                          float *pot, uint32_t *nint, int *err, cudaStream_t st) {
+                          float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st) {
     static int blocks_per_sm = 0;  // resident blocks (one persistent wave)
     if (!blocks_per_sm) {
         int b = 0;
@@ -2392,11 +2404,12 @@ int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 
             b = 1;
         blocks_per_sm = b;
     }
-    k_walk_batch_few<<<(unsigned)(c->num_sms * blocks_per_sm), kFewWarps * 32, 0, st>>>(
-        static_cast<const BatchReq *>(reqs), groups, n_groups, (group_size + 1) / 2, next, sidx, slot, a_old, acc, pot,
-        nint, err);
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg = beside_config((unsigned)(c->num_sms * blocks_per_sm), kFewWarps * 32, &attr, st);
+    cfg.numAttrs = beside ? 1 : 0;
+    TPM_CUDA(cudaLaunchKernelEx(&cfg, k_walk_batch_few, static_cast<const BatchReq *>(reqs), groups, n_groups,
+                                (group_size + 1) / 2, next, sidx, slot, a_old, acc, pot, nint, err));
     count_launch();
-    TPM_CUDA(cudaGetLastError());
     return TPM_OK;
 }
 

@@ -101,3 +101,50 @@ def test_alone_and_in_a_mix(filler):
                                                 a_old=dev(r[2].astype(np.float32)), fp=fp)
                 np.testing.assert_array_equal(a1.cpu().numpy(), a)
                 np.testing.assert_array_equal(n1.cpu().numpy(), n)
+
+
+def test_both_walks_in_a_captured_graph():
+    """A large batch and a large plain call whose chunks go to both walks, each
+    followed at once by copies of its results: replays of the captured stream
+    give the eager call's bits (what follows waits for both walks)."""
+    import torch
+
+    import paper_1909_04667_gb300 as tpm
+
+    pos, mass = W.hernquist(200000, 9)
+    rng = np.random.default_rng(9)
+    inner = np.argsort(np.sum(pos * pos, axis=1))
+    far = rng.choice(inner[60000:], 3001, replace=False)
+    ids = np.concatenate([inner[:50000], far]).astype(np.int32)
+    fp = tpm.ForceParams(theta=0.5)
+    with tpm.Context(0) as ctx:
+        s = ctx.build_tree(dev(pos), dev(mass), tpm.BuildParams(h=0.005, leaf_bucket=8))
+        off = np.array([0, 40000, len(ids)], np.int64)
+        plan = ctx.create_plan(len(ids), 2)
+        t = dev(ids)
+        acc, copy = (torch.zeros((2, len(ids), 3), device=DEV) for _ in range(2))
+
+        def calls():
+            plan.compute_forces_batch([s, s], off, fp, t, acc[0])
+            copy[0].copy_(acc[0])
+            s.compute_forces_noalloc(t, fp=fp, acc=acc[1])
+            copy[1].copy_(acc[1])
+
+        calls()
+        torch.cuda.synchronize()
+        eager = copy.cpu().numpy().copy()
+        assert (np.linalg.norm(eager, axis=2) > 0.0).all()
+        g, st = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        st.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(st), torch.cuda.graph(g, stream=st):
+            calls()
+        torch.cuda.current_stream().wait_stream(st)
+        for _ in range(5):
+            acc.zero_()
+            copy.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(copy.cpu().numpy(), eager)
+        plan.sync_status()
+        s.sync_status()
+        plan.close()
