@@ -235,7 +235,8 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
                 return TPM_EINVAL;
             }
             // groups of 64 have a walk of their own (two particles per lane)
-            const int rule = pl->group_size <= 32 ? batch_few_rule(p, offsets[r + 1] - offsets[r], n_ids) : kFewNone;
+            const int rule =
+                pl->group_size <= 32 ? batch_few_rule(s, p, offsets[r + 1] - offsets[r], n_ids) : (int)kFewNone;
             any_few = any_few || rule != kFewNone;
             all_few = all_few && rule == kFewAll;
             pl->kreq_host[r] = KeyReq{s->rank, s->n, rule};

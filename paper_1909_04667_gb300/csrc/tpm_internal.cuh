@@ -262,7 +262,7 @@ __device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__
 }
 #endif
 size_t batch_req_bytes();
-int batch_few_rule(const tpm_force_params *p, int64_t n_ids, int64_t batch_ids);
+int batch_few_rule(const System *s, const tpm_force_params *p, int64_t n_ids, int64_t batch_ids);
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
                           unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
                           float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st);

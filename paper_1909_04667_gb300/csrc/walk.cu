@@ -2413,11 +2413,8 @@ int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 
     return TPM_OK;
 }
 
-int batch_few_rule(const tpm_force_params *p, int64_t n_ids, int64_t batch_ids) {
-    if (walk_override() != 0)
-        return kFewNone;
-    const bool rel = p->crit == TPM_CRIT_RELATIVE;
-    return batch_ids <= kFewBatch ? few_rule(rel, true, n_ids) : few_span(rel, n_ids);
+int batch_few_rule(const System *s, const tpm_force_params *p, int64_t n_ids, int64_t batch_ids) {
+    return walk_override() == 0 ? few_rule_in_batch(s, p->crit == TPM_CRIT_RELATIVE, n_ids, batch_ids) : (int)kFewNone;
 }
 
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p) {

@@ -396,30 +396,38 @@ __device__ __forceinline__ void few_walk_chunk(const TreeView &T, const WalkCons
 //             two softenings (the mesh is kinder to this walk):
 //               32768 densest of 2^19    392 / 370   755 / 703    608 / 382
 //               65536 densest of 2^19    439 / 629   851 / 1257   650 / 580
+//             The relative criterion has longer and more uneven chains: batches
+//             with it keep this walk to kFewSmall ids where the systems have at
+//             most kFewSystem particles (5 x 16384 772 / 507, 10 x 8192 776 / 504).
 //   span > 0  larger requests of at most 2^16 ids: the chunks whose neighbours
 //             are on average at least that many particles apart in key order;
-//             closer ones keep the group walk.  Batches that fill the chip
-//             (16 requests for random ids of 2^19; group walk / this walk):
-//             span 16 4544 / 5675 us at theta = 0.5, 2265 / 2333 at alpha =
-//             0.0025; span 32 3162 / 3001, 1724 / 1285.
+//             closer ones keep the group walk.  From 4 in a plain call (65536
+//             random ids of 2^19, 2^20 at theta = 0.5 834 / 808, 967 / 845 us, at
+//             alpha = 0.0025 563 / 361, 645 / 375), and in a batch, whose other
+//             requests may fill the chip, from 20 (theta) or 10 (16 requests for
+//             random ids of 2^19: span 16 4544 / 5675 us at theta = 0.5, 2265 /
+//             2333 at alpha = 0.0025; span 32 3162 / 3001, 1724 / 1285).
 //   kFewNone  larger requests.
 // At 32 particles a group a request has the same bits in a plain call and in
-// every batch of at most kFewBatch ids, and in every larger batch; the two differ
-// by FP32 rounding.  Groups of 64 particles never come here.
+// every batch of at most kFewBatch ids, and in every batch larger than kFewSmall;
+// the two differ by FP32 rounding.  Groups of 64 particles never come here.
 // ----------------------------------------------------------------------
 constexpr int64_t kFewBH = 1 << 15;
 constexpr int64_t kFewRelative = 3 << 14;  // uniform softening, no mesh
 constexpr int64_t kFewOther = 1 << 16;     // relative criterion with the mesh or per-particle softening
 constexpr int64_t kFewBatch = 3 << 14;
+constexpr int64_t kFewSmall = 9 << 13, kFewSystem = 1 << 15;
 constexpr int64_t kFewRequest = 1 << 16;
-
-inline int few_span(bool relative, int64_t n_ids) {
-    return n_ids > kFewRequest ? (int)kFewNone : relative ? 16 : 32;
-}
 
 inline int few_rule(bool relative, bool uniform, int64_t n_act) {
     const int64_t line = !relative ? kFewBH : uniform ? kFewRelative : kFewOther;
-    return n_act <= line ? (int)kFewAll : few_span(relative, n_act);
+    return n_act <= line ? (int)kFewAll : n_act <= kFewRequest ? 4 : (int)kFewNone;
+}
+
+inline int few_rule_in_batch(const System *s, bool relative, int64_t n_ids, int64_t batch_ids) {
+    if (batch_ids <= kFewBatch || (relative && s->n <= kFewSystem && batch_ids <= kFewSmall))
+        return few_rule(relative, true, n_ids);
+    return n_ids > kFewRequest ? (int)kFewNone : relative ? 10 : 20;
 }
 
 // A call with chunks for both walks launches the group walk first and this one
