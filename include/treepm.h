@@ -279,7 +279,7 @@ typedef struct tpm_plan tpm_plan;
 #define TPM_BATCH_PRESORTED 1u
 
 /* Creates a plan for batches of at most max_ids ids in max_requests
- * requests (memory drawn from ctx's budget: about 42 B per id + 300 B per
+ * requests (memory drawn from ctx's budget: about 40 B per id + 300 B per
  * request).  Errors: TPM_EINVAL, TPM_EBUDGET, TPM_ECUDA. */
 int tpm_plan_create(tpm_ctx *ctx, int64_t max_ids, int64_t max_requests, tpm_plan **plan);
 

@@ -31,8 +31,8 @@ namespace {
 
 struct KeyReq {
     const uint32_t *rank;
-    int64_t n;
-    int64_t rule;  // which of its groups get two particles a warp (batch_few_rule)
+    uint32_t n;
+    int rule;  // which of its groups get two particles a warp (batch_few_rule)
 };
 
 struct Plan {
@@ -44,9 +44,8 @@ struct Plan {
     uint64_t *keys = nullptr, *skeys = nullptr;
     uint32_t *vals = nullptr, *slot = nullptr, *sidx = nullptr;
     uint32_t *gcnt = nullptr, *goff = nullptr;
-    uint4 *groups = nullptr, *few = nullptr;
-    unsigned *ngroups = nullptr;
-    unsigned *next = nullptr, *few_next = nullptr, *nfew = nullptr;  // three words, cleared together
+    uint4 *groups = nullptr;
+    unsigned *ngroups = nullptr, *next = nullptr;
     int *err = nullptr;
     int64_t *off_dev = nullptr;
     KeyReq *kreq_dev = nullptr;
@@ -84,7 +83,7 @@ __global__ void k_batch_keys(const KeyReq *__restrict__ kr, const int64_t *__res
     }
     const int64_t r = lo;
     uint32_t id = ids[i];
-    if (id >= (uint64_t)kr[r].n) {
+    if (id >= kr[r].n) {
         atomicOr(err, 1);
         id = 0;
     }
@@ -105,33 +104,40 @@ __global__ void k_batch_unpack(const uint64_t *__restrict__ skeys, int64_t n, ui
         sidx[i] = (uint32_t)skeys[i];
 }
 
-// Number of walk groups of at most g particles per request.
-__global__ void k_batch_gcount(const int64_t *__restrict__ off, int64_t n_req, int g, uint32_t *__restrict__ gcnt) {
+// Number of walk groups of at most g particles per request; clears the work
+// queues.
+__global__ void k_batch_gcount(const int64_t *__restrict__ off, int64_t n_req, int g, uint32_t *__restrict__ gcnt,
+                               unsigned *__restrict__ next, unsigned *__restrict__ nfew,
+                               unsigned long long *__restrict__ few_next) {
     const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (r < n_req)
         gcnt[r] = (uint32_t)((off[r + 1] - off[r] + g - 1) / g);
+    if (r == 0) {
+        *next = *nfew = 0u;
+        *few_next = 0ull;
+    }
 }
 
 // The group table of the persistent walk: (start, count, request, 0) for each
 // group of each request, from the scanned group counts; the total into
-// ngroups.  The groups that get two particles a warp go to a list of their
-// own (in any order: each is walked by itself) and are left in the table with
-// a count of 0.
+// ngroups.  The groups that get two particles a warp (1 instead of 0) are
+// listed too, in any order: each is walked by itself.
 __global__ void k_batch_groups(const int64_t *__restrict__ off, const KeyReq *__restrict__ kr,
                                const uint32_t *__restrict__ gcnt, const uint32_t *__restrict__ goff, int64_t n_req,
                                int g, const uint32_t *__restrict__ sidx, uint4 *__restrict__ groups,
-                               unsigned *__restrict__ ngroups, uint4 *__restrict__ few, unsigned *__restrict__ nfew) {
+                               unsigned *__restrict__ ngroups, uint32_t *__restrict__ few,
+                               unsigned *__restrict__ nfew) {
     const int64_t r = blockIdx.x;
     const int64_t lo = off[r], hi = off[r + 1];
     const uint32_t base = goff[r], ng = gcnt[r];
-    const int rule = (int)kr[r].rule;
+    const int rule = kr[r].rule;
     for (uint32_t q = threadIdx.x; q < ng; q += blockDim.x) {
         const int64_t start = lo + (int64_t)q * g;
         const int count = (int)min((int64_t)g, hi - start);
         const bool two = few_chunk(rule, sidx, start, count);
-        groups[base + q] = make_uint4((uint32_t)start, two ? 0u : (uint32_t)count, (uint32_t)r, 0u);
+        groups[base + q] = make_uint4((uint32_t)start, (uint32_t)count, (uint32_t)r, two ? 1u : 0u);
         if (two)
-            few[atomicAdd(nfew, 1u)] = make_uint4((uint32_t)start, (uint32_t)count, (uint32_t)r, 0u);
+            few[atomicAdd(nfew, 1u)] = base + q;
     }
     if (r == n_req - 1 && threadIdx.x == 0)
         *ngroups = base + ng;
@@ -239,7 +245,7 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
                 pl->group_size <= 32 ? batch_few_rule(s, p, offsets[r + 1] - offsets[r], n_ids) : (int)kFewNone;
             any_few = any_few || rule != kFewNone;
             all_few = all_few && rule == kFewAll;
-            pl->kreq_host[r] = KeyReq{s->rank, s->n, rule};
+            pl->kreq_host[r] = KeyReq{s->rank, (uint32_t)s->n, rule};
             fill_batch_req(pl->reqs_host + r * rb, s, p);
             pl->off_host[r] = offsets[r];
         }
@@ -269,22 +275,27 @@ int run_batch(Ctx *c, Plan *pl, int64_t n_req, const tpm_sys *systems, const int
         count_launch();
     }
     const int g = pl->group_size;
-    k_batch_gcount<<<(unsigned)((n_req + 255) / 256), 256, 0, st>>>(pl->off_dev, n_req, g, pl->gcnt);
+    // the list of groups that get two particles a warp, at most one per id, and
+    // its counters lie in what the sort by request has done with
+    uint32_t *few = pl->vals;
+    auto *few_next = reinterpret_cast<unsigned long long *>(pl->keys);
+    unsigned *nfew = reinterpret_cast<unsigned *>(pl->skeys);
+    k_batch_gcount<<<(unsigned)((n_req + 255) / 256), 256, 0, st>>>(pl->off_dev, n_req, g, pl->gcnt, pl->next, nfew,
+                                                                   few_next);
     count_launch();
     size_t b = pl->cub_bytes;
     TPM_CUDA(cub::DeviceScan::ExclusiveSum(pl->cub_tmp, b, pl->gcnt, pl->goff, (int)n_req, st));
     count_cub_call();
-    TPM_CUDA(cudaMemsetAsync(pl->next, 0, 3 * sizeof(unsigned), st));  // next, few_next, nfew
     k_batch_groups<<<(unsigned)n_req, 128, 0, st>>>(pl->off_dev, pl->kreq_dev, pl->gcnt, pl->goff, n_req, g, pl->sidx,
-                                                    pl->groups, pl->ngroups, pl->few, pl->nfew);
+                                                    pl->groups, pl->ngroups, few, nfew);
     count_launch();
     TPM_CUDA(cudaGetLastError());
     if (!all_few)
         TPM_CHECK(launch_walk_batch(c, g, pl->stack_depth, pl->reqs_dev, pl->groups, pl->ngroups, pl->next, pl->sidx,
                                     pl->slot, a_old, acc, pot, nint, pl->err, st));
     if (any_few)
-        TPM_CHECK(launch_walk_batch_few(c, g, pl->reqs_dev, pl->few, pl->nfew, pl->few_next, pl->sidx, pl->slot,
-                                        a_old, acc, pot, nint, pl->err, !all_few, st));
+        TPM_CHECK(launch_walk_batch_few(c, g, pl->reqs_dev, pl->groups, few, nfew, few_next, pl->sidx, pl->slot, a_old,
+                                        acc, pot, nint, pl->err, !all_few, st));
     return TPM_OK;
 }
 
@@ -327,14 +338,11 @@ int tpm_plan_create(tpm_ctx *h, int64_t max_ids, int64_t max_requests, tpm_plan 
         (rc = pl->mem.get(&pl->vals, max_ids, st)) || (rc = pl->mem.get(&pl->slot, max_ids, st)) ||
         (rc = pl->mem.get(&pl->sidx, max_ids, st)) || (rc = pl->mem.get(&pl->gcnt, max_requests, st)) ||
         (rc = pl->mem.get(&pl->goff, max_requests, st)) || (rc = pl->mem.get(&pl->groups, pl->max_groups, st)) ||
-        (rc = pl->mem.get(&pl->few, pl->max_groups, st)) || (rc = pl->mem.get(&pl->ngroups, 1, st)) ||
-        (rc = pl->mem.get(&pl->next, 3, st)) ||
+        (rc = pl->mem.get(&pl->ngroups, 1, st)) || (rc = pl->mem.get(&pl->next, 1, st)) ||
         (rc = pl->mem.get(&pl->err, 1, st)) || (rc = pl->mem.get(&pl->off_dev, max_requests + 1, st)) ||
         (rc = pl->mem.get(&pl->kreq_dev, max_requests, st)) ||
         (rc = pl->mem.get(&pl->reqs_dev, max_requests * rb, st)))
         return fail(rc);
-    pl->few_next = pl->next + 1;
-    pl->nfew = pl->next + 2;
     size_t sort_b = 0, scan_b = 0;
     if (cub::DeviceRadixSort::SortPairs(nullptr, sort_b, pl->keys, pl->skeys, pl->vals, pl->slot, (int)max_ids, 0,
                                         end_bit_for(max_requests), st) != cudaSuccess ||

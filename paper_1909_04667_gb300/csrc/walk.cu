@@ -2158,7 +2158,7 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 7)
         if (g >= total)
             break;
         const uint4 G = groups[g];
-        if (G.y == 0u)
+        if (G.w)
             continue;  // walked two particles a warp
         {
             static_assert(sizeof(BatchReq) % 4 == 0, "request records copy as words");
@@ -2182,24 +2182,24 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 7)
 // items of two particles from their own queue.
 __global__ void __launch_bounds__(kFewWarps * 32)
     k_walk_batch_few(const BatchReq *__restrict__ reqs, const uint4 *__restrict__ groups,
-                     const unsigned *__restrict__ n_groups, int items, unsigned *__restrict__ next,
-                     const uint32_t *__restrict__ sidx, const uint32_t *__restrict__ slot,
-                     const float *__restrict__ a_old, float *__restrict__ acc, float *__restrict__ pot,
-                     uint32_t *__restrict__ nint, int *__restrict__ err) {
+                     const uint32_t *__restrict__ list, const unsigned *__restrict__ listed, int items,
+                     unsigned long long *__restrict__ next, const uint32_t *__restrict__ sidx,
+                     const uint32_t *__restrict__ slot, const float *__restrict__ a_old, float *__restrict__ acc,
+                     float *__restrict__ pot, uint32_t *__restrict__ nint, int *__restrict__ err) {
     __shared__ FewShared shared[kFewWarps];
     __shared__ __align__(16) BatchReq breq[kFewWarps];
     FewShared &sh = shared[threadIdx.x >> 5];
     BatchReq &R = breq[threadIdx.x >> 5];
     const int lane = threadIdx.x & 31;
-    const unsigned long long total = (unsigned long long)*n_groups * items;
+    const unsigned long long total = (unsigned long long)*listed * items;  // may pass 2^32
     for (;;) {
-        unsigned g = 0;
+        unsigned long long g = 0;
         if (lane == 0)
-            g = atomicAdd(next, 1u);
+            g = atomicAdd(next, 1ull);
         g = __shfl_sync(0xffffffffu, g, 0);
         if (g >= total)
             break;
-        const uint4 G = groups[g / items];
+        const uint4 G = groups[list[g / items]];
         const int lo = 2 * (int)(g % items), hi = min(lo + 2, (int)G.y);
         if (lo >= hi)
             continue;
@@ -2393,8 +2393,8 @@ void set_ewald(WalkConsts &k, const System *s, const float4 *tab, float phi0) {
 
 size_t batch_req_bytes() { return sizeof(BatchReq); }
 
-int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const unsigned *n_groups,
-                          unsigned *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
+int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const uint32_t *list,
+                          const unsigned *listed, unsigned long long *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
                           float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st) {
     static int blocks_per_sm = 0;  // resident blocks (one persistent wave)
     if (!blocks_per_sm) {
@@ -2407,7 +2407,7 @@ int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 
     cudaLaunchAttribute attr;
     cudaLaunchConfig_t cfg = beside_config((unsigned)(c->num_sms * blocks_per_sm), kFewWarps * 32, &attr, st);
     cfg.numAttrs = beside ? 1 : 0;
-    TPM_CUDA(cudaLaunchKernelEx(&cfg, k_walk_batch_few, static_cast<const BatchReq *>(reqs), groups, n_groups,
+    TPM_CUDA(cudaLaunchKernelEx(&cfg, k_walk_batch_few, static_cast<const BatchReq *>(reqs), groups, list, listed,
                                 (group_size + 1) / 2, next, sidx, slot, a_old, acc, pot, nint, err));
     count_launch();
     return TPM_OK;
