@@ -134,7 +134,7 @@ __global__ void k_prepare(const double *__restrict__ pin, const float *__restric
             if (periodic) {
                 bad |= vb < box_bits || vb == minus0 ? 0 : 2;
                 v = __dadd_rn(v, sh[a]);
-                if ((uint64_t)__double_as_longlong(v) >= box_bits)
+                if (__double_as_longlong(v) >= (long long)box_bits)  // signed: -0.0 stays below
                     v = __dsub_rn(v, box);
             } else {
                 lo[a] = min(lo[a], ordered_bits(v));
