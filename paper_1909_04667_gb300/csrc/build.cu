@@ -928,8 +928,9 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     }
     for (int a = 0; a < 3; a++) {
         s->x0[a] = hst->x0[a];
-        s->bb_lo[a] = from_ordered_bits(hst->bbox[a]);
-        s->bb_hi[a] = from_ordered_bits(hst->bbox[3 + a]);
+        // a periodic build takes no bounding box: the positions' region is the box
+        s->bb_lo[a] = s->bp.periodic ? 0.0 : from_ordered_bits(hst->bbox[a]);
+        s->bb_hi[a] = s->bp.periodic ? s->bp.box : from_ordered_bits(hst->bbox[3 + a]);
     }
     s->L0 = hst->L0;
     const int64_t nn = hst->total;

@@ -164,7 +164,7 @@ struct System {
     // walk's candidate stack overflowed (read and cleared by tpm_sync_status)
     int *err = nullptr;
 
-    double bb_lo[3] = {0, 0, 0}, bb_hi[3] = {0, 0, 0};  // bounding box of the tree positions
+    double bb_lo[3] = {0, 0, 0}, bb_hi[3] = {0, 0, 0};  // bounding box of the tree positions (periodic: the box)
 
     // long-range mesh: potential and x, y, z force meshes of pm_mesh^3 points
     // (pm_mesh = pm_n, or 2 pm_n zero-padded for open boundaries) at
