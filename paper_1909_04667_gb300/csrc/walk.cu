@@ -23,6 +23,7 @@
 // a sum of small, accurately rounded terms and the pair arithmetic runs in
 // FP32 with FP32 accumulation.
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -2358,7 +2359,9 @@ int walk_override() {
 WalkConsts make_consts(const System *s, const tpm_force_params *p) {
     WalkConsts k{};
     const double h = s->bp.h;
-    k.h2 = (float)(h * h);
+    // at least the smallest normal FP32 number: masked terms (a target's own
+    // among them) are taken at r = h with mass 0, which has to give 0
+    k.h2 = std::max((float)(h * h), FLT_MIN);
     k.hinv = (float)(1.0 / h);
     k.hinv3 = (float)(1.0 / (h * h * h));
     k.thr_const = (float)(p->theta * p->theta);
