@@ -2294,10 +2294,7 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
                 s->perm, s->pos,  s->x0[0], s->x0[1],  s->x0[2], s->L0};
     if constexpr (P && T) {
         if (box) {
-            // warps per chunk: four while they fit the chip about once, two up
-            // to twice (steps with 1 / 2 / 4: 40^3 0.98 / 0.82 / 0.78 ms, 52^3
-            // 0.84 / 0.82 / 0.85, 64^3 2.16 / 2.07 / 2.04, 80^3 2.61 / 2.66 / 2.82)
-            const int split = warps <= 24 * (int64_t)num_sms ? 4 : warps <= 64 * (int64_t)num_sms ? 2 : 1;
+            const int split = box_split(warps, num_sms);
             // cell sides are the box halved: the largest not above the cutoff
             int level = 0;
             while (ldexp(s->L0, -level) > std::sqrt((double)k.rcut2) && level < kMaxLevel)
@@ -2344,9 +2341,10 @@ void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lan
 
 // Kernel choice: the group walk for open boundaries (with or without the
 // TreePM split; two targets a warp where few_rule says so), the box walk for
-// the periodic short-range walk, the lane walk for the Ewald tree (its gathers
-// want neighbouring targets in a warp's lanes).  TPM_WALK=lanes or group
-// forces one of those for comparison; all make the same per-particle decisions.
+// the periodic short-range walk (the lane walk where box_rule says so), the lane
+// walk for the Ewald tree (its gathers want neighbouring targets in a warp's
+// lanes).  TPM_WALK=lanes or group forces one of those for comparison; all make
+// the same per-particle decisions.
 int walk_override() {
     static int v = -1;
     if (v < 0) {
@@ -2522,8 +2520,8 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
         set_ewald(k, s, tab, phi0);
     }
     const int ov = walk_override();
-    const bool box = ov == 0 && per && tpm;
-    const bool lanes = ov == 1 || (ov == 0 && per && !tpm);
+    const bool box = ov == 0 && per && tpm && box_rule(s, r.n_act, rel, c->num_sms);
+    const bool lanes = ov == 1 || (ov == 0 && per && !box);
     int *err = s->err;
     if (!per && lanes) {  // the lane walk's list of cut chunks' runs: n_act entries at most
         if (!r.runs || !r.nruns) {

@@ -26,7 +26,29 @@
 // each goes on into its share of those, dealt by node index, and the first
 // alone takes what lies above (40^3 box with the spectral gradient, a step:
 // 0.95 -> 0.76 ms).
+//
+// Leaves of a particle or two (more nodes than half the particles) leave little
+// to hold against the box: a lane of the candidates, and a turn of the warp,
+// for each.  Calls that fill the chip then keep the lane walk (box_rule): steps
+// of its walk and of this one with leaf bucket 4, relative criterion, 56^3 (0.91
+// nodes a particle) 903 / 981 us, 72^3 (0.82) 2247 / 2416, 120^3 (1.03) 7124 /
+// 8188; theta = 0.5 64^3 (1.06) 1478 / 1343, 90^3 (0.63) 3271 / 3176, 110^3
+// (0.86) 3970 / 4135, 120^3 5948 / 6261.  With four warps a group this walk is
+// ahead all the same (40^3, bucket 4, relative 838 / 578).
 constexpr int kBoxWarps = 4;
+
+inline int box_split(int64_t groups, int num_sms) {
+    // warps per chunk: four while they fit the chip about once, two up to twice
+    // (steps with 1 / 2 / 4: 40^3 0.98 / 0.82 / 0.78 ms, 52^3 0.84 / 0.82 / 0.85,
+    // 64^3 2.16 / 2.07 / 2.04, 80^3 2.61 / 2.66 / 2.82)
+    return groups <= 24 * (int64_t)num_sms ? 4 : groups <= 64 * (int64_t)num_sms ? 2 : 1;
+}
+
+inline bool box_rule(const System *s, int64_t n_act, bool relative, int num_sms) {
+    const int64_t groups = (n_act + 31) / 32;
+    return 2 * s->nnodes <= s->n || groups <= (relative ? 24 : 200) * (int64_t)num_sms;
+}
+
 constexpr int kBoxStack = 384;  // child ranges, as in the walk with two targets per warp
 constexpr int kBoxSafe = kBoxStack - 64;
 
