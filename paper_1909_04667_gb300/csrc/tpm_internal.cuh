@@ -249,10 +249,11 @@ int walk_device(Ctx *c, const System *s, const tpm_force_params *p, const WalkRe
 // stack_depth is the candidate-stack capacity of the walk (128, 192 or 256).
 // The groups that get two particles a warp (few_chunk, by the rule of their
 // request: batch_few_rule for its ids and the batch's) are marked (1 instead of
-// 0) and have a list, of places in the table, and a launch of their own.  A rule above 0 is the smallest distance in key order between
+// 0) and have a list, of places in the table, and a launch of their own
+// (beside: the launch directly follows launch_walk_batch's in the stream and may
+// overlap it).  A rule above 0 is the smallest distance in key order between
 // neighbours, on average over the group; a lone particle has no neighbour and
-// would cost a whole group's chain.  beside: the launch directly follows
-// launch_walk_batch's in the stream and may overlap it.
+// would cost a whole group's chain.
 enum { kFewAll = -1, kFewNone = 0 };
 #ifdef __CUDACC__
 __device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__ sidx, int64_t g0, int gcount) {
@@ -264,8 +265,9 @@ __device__ __forceinline__ bool few_chunk(int rule, const uint32_t *__restrict__
 size_t batch_req_bytes();
 int batch_few_rule(const System *s, const tpm_force_params *p, int64_t n_ids, int64_t batch_ids);
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const uint32_t *list,
-                          const unsigned *listed, unsigned long long *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
-                          float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st);
+                          const unsigned *listed, unsigned long long *next, const uint32_t *sidx,
+                          const uint32_t *slot, const float *a_old, float *acc, float *pot, uint32_t *nint, int *err,
+                          bool beside, cudaStream_t st);
 void fill_batch_req(void *dst, const System *s, const tpm_force_params *p);
 int launch_walk_batch(Ctx *c, int group_size, int stack_depth, const void *reqs, const uint4 *groups,
                       const unsigned *n_groups, unsigned *next, const uint32_t *sidx, const uint32_t *slot,

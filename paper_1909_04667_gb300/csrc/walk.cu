@@ -440,105 +440,105 @@ __global__ void __launch_bounds__(SPLIT ? 32 * kSplitMax : kWalkThreads)
     float4 ec = make_float4(0.f, 0.f, 0.f, 0.f);  // compensation of the Ewald sums
     uint32_t cnt = 0;
     for (int seg = w; seg < (SPLIT ? warps * kSplitSegments : 1); seg += warps) {
-    const int segs = warps * kSplitSegments;
-    const int first = SPLIT ? (int)((int64_t)nnodes * seg / segs) : 0;
-    const int last = SPLIT ? (int)((int64_t)nnodes * (seg + 1) / segs) : nnodes;
-    int skip_until = valid ? 0 : 0x7fffffff;
-    int n = 0;
-    while (n < last) {
-        if (SPLIT && n < first) {
-            const int end = __ldg(&nlink[n].x);
-            if (end <= first) {  // a subtree before the segment
-                n = end;
-                continue;
-            }
-        }
-        const bool own = !SPLIT || n >= first;
-        const float4 C = __ldg(&ncen[n]);
-        const float4 O = __ldg(&ncom[n]);
-        const int4 Lk = __ldg(&nlink[n]);
-        const bool act = n >= skip_until;
-        const float dcx = C.x - gcx, dcy = C.y - gcy, dcz = C.z - gcz;  // exact
-        float px = xox - dcx, py = xoy - dcy, pz = xoz - dcz;  // particle relative to node centre
-        if (PERIODIC) {  // nearest image of the node centre as seen from this particle
-            px = wrap_min_image(px, k);
-            py = wrap_min_image(py, k);
-            pz = wrap_min_image(pz, k);
-        }
-        const float L = C.w;
-        float rx = O.x - px, ry = O.y - py, rz = O.z - pz;  // particle -> centre of mass
-        if (PERIODIC && (EWALD || L > k.bigL)) {  // the Ewald table needs the nearest image
-            rx = wrap_min_image(rx, k);
-            ry = wrap_min_image(ry, k);
-            rz = wrap_min_image(rz, k);
-        }
-        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-        bool far = false;
-        if (TREEPM) {
-            const float ex = fmaxf(fabsf(px) - 0.5f * L, 0.0f), ey = fmaxf(fabsf(py) - 0.5f * L, 0.0f),
-                        ez = fmaxf(fabsf(pz) - 0.5f * L, 0.0f);
-            far = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > k.rcut2;
-        }
-        const float gl = 0.6f * L;
-        const bool guard = k.box_guard && fabsf(px) <= gl && fabsf(py) <= gl && fabsf(pz) <= gl;
-        bool crit;
-        if (RELATIVE)
-            crit = O.w * L * L > thr * r2 * r2;
-        else
-            crit = L * L > thr * r2;
-        float hn = 0.0f;
-        if (VARH) {  // Sec. 3.2: a node of mixed softenings is opened inside its largest one
-            const float v = __ldg(&nsoft[n]);
-            hn = fabsf(v);
-            crit = crit || (v < 0.0f && hi < hn && r2 < hn * hn);
-        }
-        const bool open = act && !far && (guard || crit);
-        if (act && !open) {
-            if (!far && own) {
-                if (EWALD)
-                    ewald_pair_term(rx, ry, rz, r2, O.w, k, ax, ay, az, ph, ec);
-                else if (VARH)
-                    pair_term_h<TREEPM>(rx, ry, rz, r2, O.w, fmaxf(hi, hn), k, ax, ay, az, ph);
-                else
-                    pair_term<TREEPM>(rx, ry, rz, r2, O.w, k, ax, ay, az, ph);
-                cnt++;
-            }
-            skip_until = Lk.x;
-        }
-        const unsigned want = __ballot_sync(0xffffffffu, open);
-        if (want == 0u) {
-            n = Lk.x;
-            continue;
-        }
-        if (!Lk.w) {
-            n = n + 1;  // first child follows in pre-order
-            continue;
-        }
-        // opened leaf: particle by particle
-        const int jend = Lk.y + Lk.z;
-        for (int jj = Lk.y; jj < jend; jj++) {
-            const float4 P = __ldg(&spart[jj]);
-            if (open && (uint32_t)jj != s) {
-                float qx = P.x - px, qy = P.y - py, qz = P.z - pz;
-                if (PERIODIC && (EWALD || L > k.bigL)) {
-                    qx = wrap_min_image(qx, k);
-                    qy = wrap_min_image(qy, k);
-                    qz = wrap_min_image(qz, k);
+        const int segs = warps * kSplitSegments;
+        const int first = SPLIT ? (int)((int64_t)nnodes * seg / segs) : 0;
+        const int last = SPLIT ? (int)((int64_t)nnodes * (seg + 1) / segs) : nnodes;
+        int skip_until = valid ? 0 : 0x7fffffff;
+        int n = 0;
+        while (n < last) {
+            if (SPLIT && n < first) {
+                const int end = __ldg(&nlink[n].x);
+                if (end <= first) {  // a subtree before the segment
+                    n = end;
+                    continue;
                 }
-                const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-                if (!TREEPM || q2 <= k.rcut2) {
+            }
+            const bool own = !SPLIT || n >= first;
+            const float4 C = __ldg(&ncen[n]);
+            const float4 O = __ldg(&ncom[n]);
+            const int4 Lk = __ldg(&nlink[n]);
+            const bool act = n >= skip_until;
+            const float dcx = C.x - gcx, dcy = C.y - gcy, dcz = C.z - gcz;  // exact
+            float px = xox - dcx, py = xoy - dcy, pz = xoz - dcz;  // particle relative to node centre
+            if (PERIODIC) {  // nearest image of the node centre as seen from this particle
+                px = wrap_min_image(px, k);
+                py = wrap_min_image(py, k);
+                pz = wrap_min_image(pz, k);
+            }
+            const float L = C.w;
+            float rx = O.x - px, ry = O.y - py, rz = O.z - pz;  // particle -> centre of mass
+            if (PERIODIC && (EWALD || L > k.bigL)) {  // the Ewald table needs the nearest image
+                rx = wrap_min_image(rx, k);
+                ry = wrap_min_image(ry, k);
+                rz = wrap_min_image(rz, k);
+            }
+            const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+            bool far = false;
+            if (TREEPM) {
+                const float ex = fmaxf(fabsf(px) - 0.5f * L, 0.0f), ey = fmaxf(fabsf(py) - 0.5f * L, 0.0f),
+                            ez = fmaxf(fabsf(pz) - 0.5f * L, 0.0f);
+                far = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > k.rcut2;
+            }
+            const float gl = 0.6f * L;
+            const bool guard = k.box_guard && fabsf(px) <= gl && fabsf(py) <= gl && fabsf(pz) <= gl;
+            bool crit;
+            if (RELATIVE)
+                crit = O.w * L * L > thr * r2 * r2;
+            else
+                crit = L * L > thr * r2;
+            float hn = 0.0f;
+            if (VARH) {  // Sec. 3.2: a node of mixed softenings is opened inside its largest one
+                const float v = __ldg(&nsoft[n]);
+                hn = fabsf(v);
+                crit = crit || (v < 0.0f && hi < hn && r2 < hn * hn);
+            }
+            const bool open = act && !far && (guard || crit);
+            if (act && !open) {
+                if (!far && own) {
                     if (EWALD)
-                        ewald_pair_term(qx, qy, qz, q2, P.w, k, ax, ay, az, ph, ec);
+                        ewald_pair_term(rx, ry, rz, r2, O.w, k, ax, ay, az, ph, ec);
                     else if (VARH)
-                        pair_term_h<TREEPM>(qx, qy, qz, q2, P.w, fmaxf(hi, __ldg(&psoft[jj])), k, ax, ay, az, ph);
+                        pair_term_h<TREEPM>(rx, ry, rz, r2, O.w, fmaxf(hi, hn), k, ax, ay, az, ph);
                     else
-                        pair_term<TREEPM>(qx, qy, qz, q2, P.w, k, ax, ay, az, ph);
+                        pair_term<TREEPM>(rx, ry, rz, r2, O.w, k, ax, ay, az, ph);
                     cnt++;
                 }
+                skip_until = Lk.x;
             }
+            const unsigned want = __ballot_sync(0xffffffffu, open);
+            if (want == 0u) {
+                n = Lk.x;
+                continue;
+            }
+            if (!Lk.w) {
+                n = n + 1;  // first child follows in pre-order
+                continue;
+            }
+            // opened leaf: particle by particle
+            const int jend = Lk.y + Lk.z;
+            for (int jj = Lk.y; jj < jend; jj++) {
+                const float4 P = __ldg(&spart[jj]);
+                if (open && (uint32_t)jj != s) {
+                    float qx = P.x - px, qy = P.y - py, qz = P.z - pz;
+                    if (PERIODIC && (EWALD || L > k.bigL)) {
+                        qx = wrap_min_image(qx, k);
+                        qy = wrap_min_image(qy, k);
+                        qz = wrap_min_image(qz, k);
+                    }
+                    const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
+                    if (!TREEPM || q2 <= k.rcut2) {
+                        if (EWALD)
+                            ewald_pair_term(qx, qy, qz, q2, P.w, k, ax, ay, az, ph, ec);
+                        else if (VARH)
+                            pair_term_h<TREEPM>(qx, qy, qz, q2, P.w, fmaxf(hi, __ldg(&psoft[jj])), k, ax, ay, az, ph);
+                        else
+                            pair_term<TREEPM>(qx, qy, qz, q2, P.w, k, ax, ay, az, ph);
+                        cnt++;
+                    }
+                }
+            }
+            n = Lk.x;
         }
-        n = Lk.x;
-    }
     }
     if (SPLIT) {
         // the parts of the chunk's warps, added in FP64 (the parts are of the
@@ -859,9 +859,10 @@ __device__ __forceinline__ void sweep_pairs(const SH &sh, int e0, int e1, unsign
 // With one softening length h every entry first gets the Newtonian term at
 // max(r, h); when some lane met an entry closer than h (its smallest r^2 is
 // below h^2, rare for accepted nodes), a second pass takes the h-term of those
-// entries out again and adds their spline term.  With per-particle softening
-// (VARH) the support of an entry is the larger of the lane's own (hi) and the
-// node's largest (Sec. 3.2), and such entries add zero mass in the first pass.
+// entries out again and adds their spline term.  The mesh split and per-particle
+// softening (VARH), where an entry's support is the larger of the lane's own
+// (hi) and the node's largest (Sec. 3.2), do the same in sweep_pairs, whose
+// second pass adds the difference of the two terms.
 template <bool PERIODIC, bool TREEPM, bool VARH, class SH>
 __device__ __forceinline__ void sweep_full(const SH &sh, int nf, float xox, float xoy, float xoz, float hi,
                                            const WalkConsts &k, float &ax, float &ay, float &az, float &ph,
@@ -883,60 +884,55 @@ __device__ __forceinline__ void sweep_full(const SH &sh, int nf, float xox, floa
             const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
             if (PERIODIC && !TREEPM)
                 ewald_pair_term(rx, ry, rz, r2, A.w, k, ax, ay, az, ph, ec);
-            else if (VARH)
-                pair_term_h<TREEPM>(rx, ry, rz, r2, A.w, fmaxf(hi, sh.nsoft[e]), k, ax, ay, az, ph);
             else
                 pair_term<TREEPM>(rx, ry, rz, r2, A.w, k, ax, ay, az, ph);
         }
         return;
     }
-    if (!VARH) {
-        // pairs of entries through the two-wide FP32 instructions, each
-        // element rounded as the scalar instruction would round it; the two
-        // halves of each sum are added at the end
-        float rmin = __int_as_float(0x7f800000);
-        const float2 nx = make_float2(-xox, -xox), ny = make_float2(-xoy, -xoy), nz = make_float2(-xoz, -xoz);
-        float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
-        int e = 0;
+    // pairs of entries through the two-wide FP32 instructions, each
+    // element rounded as the scalar instruction would round it; the two
+    // halves of each sum are added at the end
+    float rmin = __int_as_float(0x7f800000);
+    const float2 nx = make_float2(-xox, -xox), ny = make_float2(-xoy, -xoy), nz = make_float2(-xoz, -xoz);
+    float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
+    int e = 0;
 #pragma unroll 2
-        for (; e + 1 < nf; e += 2) {
-            const float4 XY = sh.nxy[e >> 1], ZM = sh.nzm[e >> 1];
-            const float2 rx = __fadd2_rn(make_float2(XY.x, XY.y), nx);
-            const float2 ry = __fadd2_rn(make_float2(XY.z, XY.w), ny);
-            const float2 rz = __fadd2_rn(make_float2(ZM.x, ZM.y), nz);
-            const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
-            rmin = fminf(rmin, fminf(r2.x, r2.y));
-            const float2 ri = make_float2(rsqrtf(fmaxf(r2.x, k.h2)), rsqrtf(fmaxf(r2.y, k.h2)));
-            const float2 mr = __fmul2_rn(make_float2(ZM.z, ZM.w), ri);
-            const float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
-            sx = __ffma2_rn(mr3, rx, sx);
-            sy = __ffma2_rn(mr3, ry, sy);
-            sz = __ffma2_rn(mr3, rz, sz);
-            sp = __fadd2_rn(sp, mr);
-        }
-        ax += sx.x + sx.y;
-        ay += sy.x + sy.y;
-        az += sz.x + sz.y;
-        ph -= sp.x + sp.y;
-        for (; e < nf; e++) {
-            const float4 A = node_entry(sh, e);
+    for (; e + 1 < nf; e += 2) {
+        const float4 XY = sh.nxy[e >> 1], ZM = sh.nzm[e >> 1];
+        const float2 rx = __fadd2_rn(make_float2(XY.x, XY.y), nx);
+        const float2 ry = __fadd2_rn(make_float2(XY.z, XY.w), ny);
+        const float2 rz = __fadd2_rn(make_float2(ZM.x, ZM.y), nz);
+        const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+        rmin = fminf(rmin, fminf(r2.x, r2.y));
+        const float2 ri = make_float2(rsqrtf(fmaxf(r2.x, k.h2)), rsqrtf(fmaxf(r2.y, k.h2)));
+        const float2 mr = __fmul2_rn(make_float2(ZM.z, ZM.w), ri);
+        const float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
+        sx = __ffma2_rn(mr3, rx, sx);
+        sy = __ffma2_rn(mr3, ry, sy);
+        sz = __ffma2_rn(mr3, rz, sz);
+        sp = __fadd2_rn(sp, mr);
+    }
+    ax += sx.x + sx.y;
+    ay += sy.x + sy.y;
+    az += sz.x + sz.y;
+    ph -= sp.x + sp.y;
+    for (; e < nf; e++) {
+        const float4 A = node_entry(sh, e);
+        const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
+        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+        rmin = fminf(rmin, r2);
+        newton_term(rx, ry, rz, fmaxf(r2, k.h2), A.w, ax, ay, az, ph);
+    }
+    if (__any_sync(0xffffffffu, rmin < k.h2)) {
+        for (int q = 0; q < nf; q++) {
+            const float4 A = node_entry(sh, q);
             const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
             const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            rmin = fminf(rmin, r2);
-            newton_term(rx, ry, rz, fmaxf(r2, k.h2), A.w, ax, ay, az, ph);
-        }
-        if (__any_sync(0xffffffffu, rmin < k.h2)) {
-            for (int q = 0; q < nf; q++) {
-                const float4 A = node_entry(sh, q);
-                const float rx = A.x - xox, ry = A.y - xoy, rz = A.z - xoz;
-                const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-                if (r2 < k.h2) {
-                    newton_term(rx, ry, rz, k.h2, -A.w, ax, ay, az, ph);
-                    pair_term<false>(rx, ry, rz, r2, A.w, k, ax, ay, az, ph);
-                }
+            if (r2 < k.h2) {
+                newton_term(rx, ry, rz, k.h2, -A.w, ax, ay, az, ph);
+                pair_term<false>(rx, ry, rz, r2, A.w, k, ax, ay, az, ph);
             }
         }
-        return;
     }
 }
 
@@ -967,64 +963,58 @@ __device__ __forceinline__ void sweep_partial(const SH &sh, int np, unsigned lan
             cnt += mine ? 1u : 0u;
             if (PERIODIC && !TREEPM)
                 ewald_pair_term(rx, ry, rz, mine ? r2 : 1.0f, mine ? E.w : 0.0f, k, ax, ay, az, ph, ec);
-            else if (VARH)
-                pair_term_h<TREEPM>(rx, ry, rz, mine ? r2 : 1.0f, mine ? E.w : 0.0f, fmaxf(hi, sh.nsoft[e]), k, ax,
-                                    ay, az, ph);
             else
                 pair_term<TREEPM>(rx, ry, rz, mine ? r2 : 1.0f, mine ? E.w : 0.0f, k, ax, ay, az, ph);
         }
         return;
     }
-    if (!VARH) {
-        float rmin = __int_as_float(0x7f800000);
-        int e = e0;
-        if (e & 1) {  // an odd first entry, then aligned pairs (kNodeCap is even)
+    float rmin = __int_as_float(0x7f800000);
+    int e = e0;
+    if (e & 1) {  // an odd first entry, then aligned pairs (kNodeCap is even)
+        const float4 E = node_entry(sh, e);
+        const bool mine = (sh.nmask[e] & lanebit) != 0u;
+        const float rx = E.x - xox, ry = E.y - xoy, rz = E.z - xoz;
+        const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
+        rmin = fminf(rmin, r2);
+        cnt += mine ? 1u : 0u;
+        newton_term(rx, ry, rz, fmaxf(r2, k.h2), mine ? E.w : 0.0f, ax, ay, az, ph);
+        e++;
+    }
+    const float2 nx = make_float2(-xox, -xox), ny = make_float2(-xoy, -xoy), nz = make_float2(-xoz, -xoz);
+    float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
+#pragma unroll 2
+    for (; e < kNodeCap; e += 2) {
+        const float4 XY = sh.nxy[e >> 1], ZM = sh.nzm[e >> 1];
+        const uint2 Mk = *reinterpret_cast<const uint2 *>(&sh.nmask[e]);
+        const bool m0 = (Mk.x & lanebit) != 0u, m1 = (Mk.y & lanebit) != 0u;
+        const float2 rx = __fadd2_rn(make_float2(XY.x, XY.y), nx);
+        const float2 ry = __fadd2_rn(make_float2(XY.z, XY.w), ny);
+        const float2 rz = __fadd2_rn(make_float2(ZM.x, ZM.y), nz);
+        const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
+        rmin = fminf(rmin, fminf(r2.x, r2.y));
+        cnt += (m0 ? 1u : 0u) + (m1 ? 1u : 0u);
+        const float2 ri = make_float2(rsqrtf(fmaxf(r2.x, k.h2)), rsqrtf(fmaxf(r2.y, k.h2)));
+        const float2 mr = __fmul2_rn(make_float2(m0 ? ZM.z : 0.0f, m1 ? ZM.w : 0.0f), ri);
+        const float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
+        sx = __ffma2_rn(mr3, rx, sx);
+        sy = __ffma2_rn(mr3, ry, sy);
+        sz = __ffma2_rn(mr3, rz, sz);
+        sp = __fadd2_rn(sp, mr);
+    }
+    ax += sx.x + sx.y;
+    ay += sy.x + sy.y;
+    az += sz.x + sz.y;
+    ph -= sp.x + sp.y;
+    if (__any_sync(0xffffffffu, rmin < k.h2)) {
+        for (int e = e0; e < kNodeCap; e++) {
             const float4 E = node_entry(sh, e);
-            const bool mine = (sh.nmask[e] & lanebit) != 0u;
             const float rx = E.x - xox, ry = E.y - xoy, rz = E.z - xoz;
             const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-            rmin = fminf(rmin, r2);
-            cnt += mine ? 1u : 0u;
-            newton_term(rx, ry, rz, fmaxf(r2, k.h2), mine ? E.w : 0.0f, ax, ay, az, ph);
-            e++;
-        }
-        const float2 nx = make_float2(-xox, -xox), ny = make_float2(-xoy, -xoy), nz = make_float2(-xoz, -xoz);
-        float2 sx = make_float2(0.f, 0.f), sy = sx, sz = sx, sp = sx;
-#pragma unroll 2
-        for (; e < kNodeCap; e += 2) {
-            const float4 XY = sh.nxy[e >> 1], ZM = sh.nzm[e >> 1];
-            const uint2 Mk = *reinterpret_cast<const uint2 *>(&sh.nmask[e]);
-            const bool m0 = (Mk.x & lanebit) != 0u, m1 = (Mk.y & lanebit) != 0u;
-            const float2 rx = __fadd2_rn(make_float2(XY.x, XY.y), nx);
-            const float2 ry = __fadd2_rn(make_float2(XY.z, XY.w), ny);
-            const float2 rz = __fadd2_rn(make_float2(ZM.x, ZM.y), nz);
-            const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __fmul2_rn(rz, rz)));
-            rmin = fminf(rmin, fminf(r2.x, r2.y));
-            cnt += (m0 ? 1u : 0u) + (m1 ? 1u : 0u);
-            const float2 ri = make_float2(rsqrtf(fmaxf(r2.x, k.h2)), rsqrtf(fmaxf(r2.y, k.h2)));
-            const float2 mr = __fmul2_rn(make_float2(m0 ? ZM.z : 0.0f, m1 ? ZM.w : 0.0f), ri);
-            const float2 mr3 = __fmul2_rn(__fmul2_rn(mr, ri), ri);
-            sx = __ffma2_rn(mr3, rx, sx);
-            sy = __ffma2_rn(mr3, ry, sy);
-            sz = __ffma2_rn(mr3, rz, sz);
-            sp = __fadd2_rn(sp, mr);
-        }
-        ax += sx.x + sx.y;
-        ay += sy.x + sy.y;
-        az += sz.x + sz.y;
-        ph -= sp.x + sp.y;
-        if (__any_sync(0xffffffffu, rmin < k.h2)) {
-            for (int e = e0; e < kNodeCap; e++) {
-                const float4 E = node_entry(sh, e);
-                const float rx = E.x - xox, ry = E.y - xoy, rz = E.z - xoz;
-                const float r2 = fmaf(rx, rx, fmaf(ry, ry, rz * rz));
-                if ((sh.nmask[e] & lanebit) && r2 < k.h2) {
-                    newton_term(rx, ry, rz, k.h2, -E.w, ax, ay, az, ph);
-                    pair_term<false>(rx, ry, rz, r2, E.w, k, ax, ay, az, ph);
-                }
+            if ((sh.nmask[e] & lanebit) && r2 < k.h2) {
+                newton_term(rx, ry, rz, k.h2, -E.w, ax, ay, az, ph);
+                pair_term<false>(rx, ry, rz, r2, E.w, k, ax, ay, az, ph);
             }
         }
-        return;
     }
 }
 
@@ -1149,8 +1139,6 @@ __device__ __forceinline__ void sweep_leaves(const SH &sh, int nl, unsigned lane
             if (mine && (uint32_t)jj != self && (!TREEPM || q2 <= k.rcut2)) {
                 if (PERIODIC && !TREEPM)
                     ewald_pair_term(qx, qy, qz, q2, P.w, k, ax, ay, az, ph, ec);
-                else if (VARH)
-                    pair_term_h<TREEPM>(qx, qy, qz, q2, P.w, fmaxf(hi, __ldg(&psoft[jj])), k, ax, ay, az, ph);
                 else
                     pair_term<TREEPM>(qx, qy, qz, q2, P.w, k, ax, ay, az, ph);
                 cnt++;
@@ -1409,11 +1397,7 @@ __device__ __forceinline__ void group_walk(const TreeView &T, const WalkConsts &
                     far = fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > k.rcut2;
                 }
                 const bool guard = k.box_guard && fabsf(px) <= gl && fabsf(py) <= gl && fabsf(pz) <= gl;
-                bool crit = RELATIVE ? (q > P.w * r2 * r2) : (q > P.w * r2);
-                if (VARH) {  // Sec. 3.2: a node of mixed softenings is opened inside its largest one
-                    const float hp = __shfl_sync(FULL, hi, p);
-                    crit = crit || (hsig < 0.0f && hp < -hsig && r2 < hsig * hsig);
-                }
+                const bool crit = RELATIVE ? (q > P.w * r2 * r2) : (q > P.w * r2);
                 const unsigned b = 1u << p;
                 if (act && !far)
                     (guard || crit) ? (om |= b) : (am |= b);
@@ -2261,8 +2245,8 @@ __global__ void __launch_bounds__(kGroupWarps * 32, 5)
 }
 
 template <bool P, bool R, bool T, bool V>
-void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, bool box, int rule, int *err, int num_sms,
-            cudaStream_t st) {
+void launch(const System *s, const WalkRequest &r, const WalkConsts &k, bool lanes, bool box, int rule, int *err,
+            int num_sms, cudaStream_t st) {
     const int64_t warps = (r.n_act + 31) / 32;
     if (lanes) {
         auto walk = [&](auto kernel, int64_t blocks, int threads, size_t smem) {
@@ -2395,8 +2379,9 @@ void set_ewald(WalkConsts &k, const System *s, const float4 *tab, float phi0) {
 size_t batch_req_bytes() { return sizeof(BatchReq); }
 
 int launch_walk_batch_few(Ctx *c, int group_size, const void *reqs, const uint4 *groups, const uint32_t *list,
-                          const unsigned *listed, unsigned long long *next, const uint32_t *sidx, const uint32_t *slot, const float *a_old, float *acc,
-                          float *pot, uint32_t *nint, int *err, bool beside, cudaStream_t st) {
+                          const unsigned *listed, unsigned long long *next, const uint32_t *sidx,
+                          const uint32_t *slot, const float *a_old, float *acc, float *pot, uint32_t *nint, int *err,
+                          bool beside, cudaStream_t st) {
     static int blocks_per_sm = 0;  // resident blocks (one persistent wave)
     if (!blocks_per_sm) {
         int b = 0;
