@@ -957,8 +957,16 @@ int build_tree_device(Ctx *c, System *s, const double *pos_in, const float *mass
     tmp_b.add(&hist, cells);
     tmp_b.add(&place, cells);
     tmp_b.add(&list, nn);
-    tmp_b.add(&late, kLevels * stretches);
-    tmp_b.add(&later, kLevels * ((stretches + kLateFan - 1) / kLateFan));
+    // the lists of nodes that reach past their stretch, by particles and not by
+    // nodes, lie in the unsorted keys, which the sort has done with (a system of
+    // few, large leaves needs no more memory for them)
+    const int64_t late_n = kLevels * stretches, later_n = kLevels * ((stretches + kLateFan - 1) / kLateFan);
+    late = reinterpret_cast<uint32_t *>(key_raw);
+    later = late + late_n;
+    if (late_n + later_n > 2 * n) {  // n below 22
+        tmp_b.add(&late, late_n);
+        tmp_b.add(&later, later_n);
+    }
     if (place_bytes > cub_bytes)
         tmp_b.add(&place_tmp, place_bytes);
     if (s->psoft) {
