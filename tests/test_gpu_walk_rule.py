@@ -148,3 +148,28 @@ def test_both_walks_in_a_captured_graph():
         plan.sync_status()
         s.sync_status()
         plan.close()
+
+
+def test_groups_of_64_have_the_same_bits_in_any_mix():
+    """A plan with groups of 64 particles has one walk for all: what a request gets does not depend on the batch."""
+    import torch
+
+    import paper_1909_04667_gb300 as tpm
+
+    rng = np.random.default_rng(8)
+    with tpm.Context(0) as ctx:
+        pos, mass = W.plummer(70000, 8)
+        s = ctx.build_tree(dev(pos), dev(mass), tpm.BuildParams(h=0.01, leaf_bucket=8))
+        ids, rest = rng.choice(70000, 3333, replace=False).astype(np.int32), np.arange(70000, dtype=np.int32)
+        plan = ctx.create_plan(80000, 2)
+        plan.group_size = 64
+        out = []
+        for more in (rest[:0], rest[:9000], rest):
+            acc = torch.empty((len(ids) + len(more), 3), device=DEV)
+            plan.compute_forces_batch([s, s], np.array([0, len(more), len(more) + len(ids)]), tpm.ForceParams(theta=0.6),
+                                      dev(np.concatenate([more, ids])), acc)
+            plan.sync_status()
+            out.append(acc[len(more):].cpu().numpy())
+        plan.close()
+    np.testing.assert_array_equal(out[0], out[1])
+    np.testing.assert_array_equal(out[0], out[2])
