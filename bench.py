@@ -43,9 +43,9 @@ FLOPS_PER_INTERACTION = 20  # monopole pair term with potential, FP32: offset 3,
 # from: DRAM bytes (read + write) and the pipe activity of that launch (the
 # FMA pipe's busy cycles, counting the two-wide FP32 instructions, and the
 # ALU pipe's instructions, both against their peaks)
-WALK_TRAFFIC = {"bytes": 86.534912e6 + 14.030592e6,
-                "fma_pipe_active": 0.44231552, "alu_pipe_inst": 0.55374613,
-                "walk_cu_sha256": "867b744ebbf10b18da0af3149727d26d41b38cd8d6e082e20c7de0b9305b7e9f"}
+WALK_TRAFFIC = {"bytes": 86.964992e6 + 13.945088e6,
+                "fma_pipe_active": 0.44148286, "alu_pipe_inst": 0.55393982,
+                "walk_cu_sha256": "35c3bcec58bd608936e982b930efb074582d7b39580daf92f469286cc1fea0e1"}
 
 
 def walk_capture():

@@ -268,8 +268,12 @@ int tpm_compute_forces_noalloc(tpm_ctx *ctx, tpm_sys s, const uint32_t *active_i
  * sequence of batched calls can be captured in a CUDA graph.  All requests
  * of one call run in one persistent walk launch: resident warps take groups
  * of at most G consecutive (key-ordered) particles of any request from a
- * device work queue (groups of small systems, and of small requests whose
- * particles lie apart, from a second queue, two particles a warp).
+ * device work queue (those that leave the chip idle, and those whose particles
+ * lie apart, from a second queue, two particles a warp).  Every particle gets
+ * the plain call's interaction set.  At the default group size and stack depth
+ * a request also has the plain call's bits in any batch of at most 49152 ids; in
+ * larger ones its forces may differ from them by FP32 rounding (beyond 73728 ids
+ * all batches give it the same bits, as all batches do at 64 particles a group).
  * Open-boundary systems only.
  */
 typedef struct tpm_plan tpm_plan;

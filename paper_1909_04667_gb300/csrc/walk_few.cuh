@@ -433,11 +433,12 @@ inline int few_rule_in_batch(const System *s, bool relative, int64_t n_ids, int6
 // A call with chunks for both walks launches the group walk first and this one
 // right behind it in the same stream, allowed to start as soon as all blocks of
 // the group walk run (they say so with cudaTriggerProgrammaticLaunchCompletion):
-// its warps then fill what the group walk leaves idle.  Side by side on a second
-// stream, or first in line, this walk took the places that the group walk's
-// blocks spread over, and its long chains met on few SMs: 65536 random ids of
-// 2^19 in one batch, 31 of 2048 chunks for this walk, 1250 us without them, 1590
-// on a second stream, 1150 this way; 16 x 8192 of 2^16 1284, 1770 and 1270.
+// its warps then fill what the group walk leaves idle.  Beside it on a second
+// stream this walk took the places that the group walk's blocks spread over, and
+// its long chains met on few SMs.  Batches of requests for 2048 random ids of
+// 2^16 at theta = 0.5, chunks of spread 32 and more to this walk (us, groups
+// only / second stream / one after the other / this way): 64 requests 1810 / 2320
+// / 2310 / 1760, 16 requests 1650 / 1850 / 1450 / 1180.
 // Block 0 of this walk waits for the group walk before it ends, so that what
 // follows in the stream follows both.
 inline cudaLaunchConfig_t beside_config(unsigned blocks, int threads, cudaLaunchAttribute *attr, cudaStream_t st) {
